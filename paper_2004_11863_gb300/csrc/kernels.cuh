@@ -1336,13 +1336,16 @@ __global__ void __launch_bounds__(RstTile<L>::NT, HRR ? RstTile<L>::MINB_HRR : R
 }
 
 // ------------------------------------------------------ set-up / read-out
+// Node t of a level, x fastest.  32-bit division (a level has fewer than
+// 2^31 nodes: the host holds every plane below that): the 64-bit form cost
+// more instructions than a D2Q9 node's whole read-out.
 __device__ __forceinline__ bool node_of(const LevelView& v, long long t, int& x, int& y, int& z) {
   const long long N = (long long)v.n[0] * v.n[1] * v.n[2];
   if (t >= N) return false;
-  x = (int)(t % v.n[0]);
-  t /= v.n[0];
-  y = (int)(t % v.n[1]);
-  z = (int)(t / v.n[1]);
+  const unsigned u = (unsigned)t, row = u / (unsigned)v.n[0];
+  x = (int)(u - row * (unsigned)v.n[0]);
+  z = (int)(row / (unsigned)v.n[1]);
+  y = (int)(row - (unsigned)z * (unsigned)v.n[1]);
   return true;
 }
 
@@ -1397,9 +1400,7 @@ struct Acc2 {
 
 // drho = sum g and j = sum xi g (shifted populations), each through Acc2.
 template <class L>
-__device__ __forceinline__ void moments_acc(const float (&g)[L::Q], double& drho, double& jx,
-                                            double& jy, double& jz) {
-  Acc2 r, m[3];
+__device__ __forceinline__ void moments_acc2(const float (&g)[L::Q], Acc2& r, Acc2 (&m)[3]) {
   sfor<L::Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
     r.add(g[i]);
@@ -1409,6 +1410,12 @@ __device__ __forceinline__ void moments_acc(const float (&g)[L::Q], double& drho
       if (L::c(i, a) == -1) m[a].add(-g[i]);
     }
   });
+}
+template <class L>
+__device__ __forceinline__ void moments_acc(const float (&g)[L::Q], double& drho, double& jx,
+                                            double& jy, double& jz) {
+  Acc2 r, m[3];
+  moments_acc2<L>(g, r, m);
   drho = r.value();
   jx = m[0].value();
   jy = m[1].value();
@@ -1472,11 +1479,10 @@ __global__ void __launch_bounds__(kDiagThreads)
     for (int j = 0; j < 3; ++j) partial[(long long)j * gridDim.x + blockIdx.x] = sh[j][0];
 }
 
-// rho and u (FP64 or FP32 outputs) of the post-collision state; NaN at
-// inactive nodes.
-template <class L, class S, class T>
+// rho and u (FP64) of the post-collision state; NaN at inactive nodes.
+template <class L, class S>
 // (nodes t0 .. t0 + cnt - 1 into rho[t - t0], u[a * us + t - t0])
-__global__ void k_macros(LevelView v, int run, int last, T* rho, T* u, long long us,
+__global__ void k_macros(LevelView v, int run, int last, double* rho, double* u, long long us,
                          long long t0, long long cnt, RefState ref) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= cnt) return;
@@ -1484,7 +1490,7 @@ __global__ void k_macros(LevelView v, int run, int last, T* rho, T* u, long long
   int x, y, z;
   if (!node_of(v, t, x, y, z)) return;
   if (inactive(v, x, y, z)) {
-    const T nan = T(__longlong_as_double(0x7ff8000000000000ULL));
+    const double nan = __longlong_as_double(0x7ff8000000000000ULL);
     rho[k] = nan;
     u[k] = u[us + k] = u[2 * us + k] = nan;
     return;
@@ -1497,10 +1503,64 @@ __global__ void k_macros(LevelView v, int run, int last, T* rho, T* u, long long
   double drho, jx, jy, jz;
   moments_acc<L>(g, drho, jx, jy, jz);
   const double r = ref.rho0 + drho, ri = 1.0 / r;
-  rho[k] = T(r);
-  u[k] = T((jx + ref.rho0 * ref.U[0]) * ri);
-  u[us + k] = T((jy + ref.rho0 * ref.U[1]) * ri);
-  u[2 * us + k] = T(L::D == 3 ? (jz + ref.rho0 * ref.U[2]) * ri : 0.0);
+  rho[k] = r;
+  u[k] = (jx + ref.rho0 * ref.U[0]) * ri;
+  u[us + k] = (jy + ref.rho0 * ref.U[1]) * ri;
+  u[2 * us + k] = L::D == 3 ? (jz + ref.rho0 * ref.U[2]) * ri : 0.0;
+}
+
+// The reference state as unevaluated sums of two binary32 numbers (rho0 and
+// the reference momentum rho0 U), formed on the host.
+struct RefPair {
+  float r_hi, r_lo;
+  float m_hi[3], m_lo[3];
+};
+
+// rho and u of the post-collision state in binary32; NaN at inactive nodes.
+// The same values as k_macros rounded to binary32, without its FP64
+// arithmetic: every quantity stays an unevaluated binary32 pair (hi + lo, as
+// accurate as the sums of Acc2) until the one final rounding, and the
+// quotient is the rounded one plus its residual, formed exactly by an FMA,
+// over the density.  GB300 runs FP64 at a small fraction of its binary32
+// rate, so the FP64 reciprocal and products bounded the read-out: the
+// 67 M + 17 M nodes of a D3Q19 slab took 4.16 ms and take 1.40 ms (5.5 TB/s
+// of the 92 bytes a node; now bound by HBM).
+template <class L, class S>
+__global__ void __launch_bounds__(128)
+    k_macros_f(LevelView v, int run, int last, float* rho, float* u, RefPair R) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long N = (long long)v.n[0] * v.n[1] * v.n[2];
+  int x, y, z;
+  if (!node_of(v, t, x, y, z)) return;
+  if (inactive(v, x, y, z)) {
+    const float nan = __int_as_float(0x7fc00000);
+    rho[t] = u[t] = u[N + t] = u[2 * N + t] = nan;
+    return;
+  }
+  float g[L::Q];
+  load_post<L, S>(run_cptr<S>(v, run), v.plane, node_addr<L>(v, x, y, z), last, v.es, g);
+  Acc2 r, m[3];
+  moments_acc2<L>(g, r, m);
+  // rho = rho0 + drho as a pair (rh, rl): TwoSum, then one renormalisation
+  r.e += R.r_lo;
+  r.add(R.r_hi);
+  const float rh = r.s + r.e, rl = r.e - (rh - r.s);
+  rho[t] = rh;
+  const float inv = __frcp_rn(rh);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float q = 0.0f;
+    if (a < L::D) {
+      m[a].e += R.m_lo[a];
+      m[a].add(R.m_hi[a]);
+      const float nh = m[a].s + m[a].e, nl = m[a].e - (nh - m[a].s);
+      q = nh * inv;
+      const float d = (fmaf(-q, rh, nh) + fmaf(-q, rl, nl)) * inv;
+      // (no correction to an infinite or NaN quotient)
+      if (fabsf(q) < INFINITY) q += d;
+    }
+    u[a * N + t] = q;
+  }
 }
 
 // Post-collision populations shifted by the rest state, f_i - w_i rho0,

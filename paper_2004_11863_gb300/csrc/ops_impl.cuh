@@ -402,21 +402,28 @@ cudaError_t macros_d(const LevelView& v, int storage, int run, int last, double*
   if (cnt <= 0) return cudaSuccess;
   unsigned g = blocks_for(cnt, 128);
   if (storage == 0)
-    k_macros<L, float, double><<<g, 128, 0, s>>>(v, run, last, rho, u, us, t0, cnt, ref);
+    k_macros<L, float><<<g, 128, 0, s>>>(v, run, last, rho, u, us, t0, cnt, ref);
   else
-    k_macros<L, __half, double><<<g, 128, 0, s>>>(v, run, last, rho, u, us, t0, cnt, ref);
+    k_macros<L, __half><<<g, 128, 0, s>>>(v, run, last, rho, u, us, t0, cnt, ref);
   return cudaGetLastError();
 }
 
 template <class L>
 cudaError_t macros_f(const LevelView& v, int storage, int run, int last, float* rho, float* u,
                      const RefState& ref, cudaStream_t s) {
-  const long long N = nodes(v);
-  unsigned g = blocks_for(N, 128);
+  const unsigned g = blocks_for(nodes(v), 128);
+  RefPair R;
+  R.r_hi = (float)ref.rho0;
+  R.r_lo = (float)(ref.rho0 - R.r_hi);
+  for (int a = 0; a < 3; ++a) {
+    const double m = ref.rho0 * ref.U[a];
+    R.m_hi[a] = (float)m;
+    R.m_lo[a] = (float)(m - R.m_hi[a]);
+  }
   if (storage == 0)
-    k_macros<L, float, float><<<g, 128, 0, s>>>(v, run, last, rho, u, N, 0, N, ref);
+    k_macros_f<L, float><<<g, 128, 0, s>>>(v, run, last, rho, u, R);
   else
-    k_macros<L, __half, float><<<g, 128, 0, s>>>(v, run, last, rho, u, N, 0, N, ref);
+    k_macros_f<L, __half><<<g, 128, 0, s>>>(v, run, last, rho, u, R);
   return cudaGetLastError();
 }
 
