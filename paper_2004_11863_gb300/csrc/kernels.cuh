@@ -30,7 +30,6 @@
 
 #include "desc.h"
 #include "lattice.cuh"
-#include "lattice_x2.cuh"
 
 namespace mlbm {
 
@@ -373,7 +372,7 @@ __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
 
 // Level update, two nodes per thread in one two-lane collision: the nodes
 // (x, y0) and (x, y0 + 1) take the two lanes of the packed FP32 arithmetic
-// (lattice_x2.cuh), so their collisions issue about half the floating-point
+// (F2 of lattice.cuh), so their collisions issue about half the floating-point
 // instructions of two scalar collisions.  A lane whose node is outside the
 // level or inactive computes on its partner's populations and stores
 // nothing.  Per lattice, K1X2_<lattice> selects this kernel over
@@ -542,7 +541,7 @@ __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float
       });
     }
   }
-  collide_emit_x2<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
+  collide_emit<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
     constexpr int i = decltype(I)::value;
     if constexpr (PAR == 0) {
       if (ok0) Store<S>::st(&f[(X2Idx)opp<L>(i) * (X2Idx)v.plane + a0.at(0, 0, 0)], val.v.x);
@@ -609,7 +608,7 @@ __global__ void __launch_bounds__(128, std::is_same<S, float>::value
 // one thread updates one node of runs 2p and 2p+1, moving each direction of
 // both runs with one 4-byte access (a half2 of the two runs' values), and
 // computes the two collisions as one two-lane collision on the packed FP32
-// instructions (lattice_x2.cuh).  The last
+// instructions (F2 of lattice.cuh).  The last
 // pair of an odd batch carries an unused run that stays at rest (zero
 // deviations collide to zero; no interface kernel touches it).
 template <class L>
@@ -677,7 +676,7 @@ __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
       });
     }
   }
-  collide_emit_x2<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
+  collide_emit<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
     constexpr int i = decltype(I)::value;
     const __half2 h = __float22half2_rn(val.v);
     if constexpr (PAR == 0)
@@ -693,11 +692,9 @@ __device__ __forceinline__ void split_neq(const float (&g)[L::Q], const RefF& R,
                                           float& dux, float& duy, float& duz,
                                           float (&f1)[L::Q]) {
   deviations<L>(g, R, drho, dux, duy, duz);
-  float g0[L::Q];
-  equilibrium_f<L>(drho, dux, duy, duz, R, g0);
-  sfor<L::Q>([&](auto I) {
+  equilibrium_emit<L>(drho, dux, duy, duz, R, [&](auto I, float g0) {
     constexpr int i = decltype(I)::value;
-    f1[i] = g[i] - g0[i];
+    f1[i] = g[i] - g0;
   });
 }
 
@@ -815,14 +812,6 @@ template <class L, class S, int G, class V>
 __device__ __forceinline__ void inject_rebuild(const LevelView& c, int run, int x, int y, int z,
                                                int par, float resc, const RefF& ref, int grp,
                                                V val, S* xf, int xs) {
-  const float drho = val(0), dux = val(1), duy = val(2);
-  const float duz = (L::D == 3) ? val(3) : 0.0f;
-  const float Ux = ref.Ux, Uy = ref.Uy, Uz = (L::D == 3) ? ref.Uz : 0.0f;
-  const float ux = Ux + dux, uy = Uy + duy, uz = Uz + duz;
-  float A[7], dA[7];
-  third_coeffs(ux, uy, uz, dux, duy, duz, Ux, Uy, Uz, A, dA);
-  const float dusq = 1.5f * (dux * (ux + Ux) + duy * (uy + Uy) + duz * (uz + Uz));
-  const float rho = ref.rho0 + drho;
   S* fb = run_ptr<S>(c, run);
   const NodeAddr ad = node_addr<L>(c, x, y, z);
   const long long F = (long long)c.n[1] * c.n[2];
@@ -830,11 +819,11 @@ __device__ __forceinline__ void inject_rebuild(const LevelView& c, int run, int 
   if (xs >= 0)
     xb = xf + ((((long long)(run / c.es) * 2 + xs) * L::Q * F + (long long)z * c.n[1] + y) * c.es +
                run % c.es);
-  sfor<L::Q>([&](auto I) {
+  equilibrium_emit<L>(val(0), val(1), val(2), L::D == 3 ? val(3) : 0.0f, ref,
+                      [&](auto I, float g0) {
     constexpr int i = decltype(I)::value;
     if (i % G == grp) {
-      const float g = eq_i<L, i, true>(drho, rho, dux, duy, duz, dusq, dA, ref) +
-                      resc * val(4 + i);
+      const float g = g0 + resc * val(4 + i);
       if (xs >= 0)
         Store<S>::st(xb + (long long)i * F * c.es, g);
       else
@@ -1290,7 +1279,7 @@ __global__ void __launch_bounds__(RstTile<L>::NT, HRR ? RstTile<L>::MINB_HRR : R
           um[ax][b] = cu0[b][v - 1][u];
         }
       }
-    HrrIn hy;
+    HrrIn<float> hy;
     hy.sig = sig;
     hy.ks = ks_p;
     strain_from<L>(up, um, hy.s);
@@ -1315,23 +1304,13 @@ __global__ void __launch_bounds__(RstTile<L>::NT, HRR ? RstTile<L>::MINB_HRR : R
     for (int b = 0; b < L::D; ++b) dp[(long long)b * p.plane] = cm[j][i][1 + b];
     return;
   }
-  const float drho = cm[j][i][0], dux = cm[j][i][1], duy = cm[j][i][2];
-  const float duz = (L::D == 3) ? cm[j][i][3] : 0.0f;
-  const float Ux = ref.Ux, Uy = ref.Uy, Uz = (L::D == 3) ? ref.Uz : 0.0f;
-  const float ux = Ux + dux, uy = Uy + duy, uz = Uz + duz;
-  float Ac[7], dA[7];
-  third_coeffs(ux, uy, uz, dux, duy, duz, Ux, Uy, Uz, Ac, dA);
-  const float dusq = 1.5f * (dux * (ux + Ux) + duy * (uy + Uy) + duz * (uz + Uz));
-  const float rho = ref.rho0 + drho;
   S* fp = run_ptr<S>(p, run);
   const NodeAddr ad = node_addr<L>(p, pc(0), pc(1), pc(2));
-  sfor<Q>([&](auto I) {
+  equilibrium_emit<L>(cm[j][i][0], cm[j][i][1], cm[j][i][2], cm[j][i][3], ref,
+                      [&](auto I, float g0) {
     constexpr int q = decltype(I)::value;
-    if (q % TT::G == grp) {
-      const float g = eq_i<L, q, true>(drho, rho, dux, duy, duz, dusq, dA, ref) +
-                      resc * Cf[q][j][i];
-      store_pre_i<L, S, q>(fp, p.plane, ad, ppar, p.es, g);
-    }
+    if (q % TT::G == grp)
+      store_pre_i<L, S, q>(fp, p.plane, ad, ppar, p.es, g0 + resc * Cf[q][j][i]);
   });
 }
 

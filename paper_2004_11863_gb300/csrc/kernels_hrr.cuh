@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(128)
       um[ax][b] = __ldg(d + (long long)b * v.plane + em);
     }
   }
-  HrrIn hy;
+  HrrIn<float> hy;
   hy.sig = sig;
   hy.ks = ks;
   strain_from<L>(up, um, hy.s);
@@ -251,7 +251,7 @@ __global__ void k_collide_bnd(LevelView c, BndDesc B, RingDesc R, const float* s
         Sv[j] += w * vt;
       }
     }
-  HrrIn hy;
+  HrrIn<float> hy;
   hy.sig = sig;
   hy.ks = ks;
 #pragma unroll

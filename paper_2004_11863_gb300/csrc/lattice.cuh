@@ -191,50 +191,6 @@ __host__ __device__ __forceinline__ void moments(const T (&g)[L::Q], T& drho, T&
   });
 }
 
-// Moments from per-axis class sums: S+_a = sum over xi_a = +1, S-_a = sum
-// over xi_a = -1; then j_a = S+_a - S-_a and the diagonal second moment
-// P_aa = S+_a + S-_a, and drho = S+_x + S-_x + (sum over xi_x = 0).  The
-// off-diagonal P_ab sum the four directions with xi_a xi_b = +-1.
-template <class L>
-__device__ __forceinline__ void moments2(const float (&g)[L::Q], float& drho, float (&j)[3],
-                                         float (&pd)[3], float (&po)[3]) {
-  float sp[3] = {0, 0, 0}, sm[3] = {0, 0, 0}, s0 = 0.0f;
-  sfor<L::Q>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    if constexpr (L::c(i, 0) == 1) sp[0] += g[i];
-    if constexpr (L::c(i, 0) == -1) sm[0] += g[i];
-    if constexpr (L::c(i, 0) == 0) s0 += g[i];
-  });
-  sfor<L::Q>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    if constexpr (L::c(i, 1) == 1) sp[1] += g[i];
-    if constexpr (L::c(i, 1) == -1) sm[1] += g[i];
-    if constexpr (L::D == 3) {
-      if constexpr (L::c(i, 2) == 1) sp[2] += g[i];
-      if constexpr (L::c(i, 2) == -1) sm[2] += g[i];
-    }
-  });
-  drho = (sp[0] + sm[0]) + s0;
-  for (int a = 0; a < 3; ++a) {
-    j[a] = sp[a] - sm[a];
-    pd[a] = sp[a] + sm[a];
-  }
-  float pxy_p = 0, pxy_m = 0, pxz_p = 0, pxz_m = 0, pyz_p = 0, pyz_m = 0;
-  sfor<L::Q>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    constexpr int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
-    if constexpr (cx * cy == 1) pxy_p += g[i];
-    if constexpr (cx * cy == -1) pxy_m += g[i];
-    if constexpr (cx * cz == 1) pxz_p += g[i];
-    if constexpr (cx * cz == -1) pxz_m += g[i];
-    if constexpr (cy * cz == 1) pyz_p += g[i];
-    if constexpr (cy * cz == -1) pyz_m += g[i];
-  });
-  po[0] = pxy_p - pxy_m;
-  po[1] = pxz_p - pxz_m;
-  po[2] = pyz_p - pyz_m;
-}
-
 // Third-order coefficients of u (A) and their deviations from those of U
 // (dA = A(u) - A(U)), in the order [xxy, xxz, yyx, yyz, zzx, zzy, xyz].
 template <class T>
@@ -293,46 +249,351 @@ __host__ __device__ __forceinline__ void equilibrium_dev(T drho, T dux, T duy, T
   });
 }
 
-// Reference state (rho0, U) of the shifted storage, in binary32, with the
-// per-direction constants the equilibrium deviation needs:
-// c1[i] = 1 + e_i(U) and cU2[i] = 2 xi_i.U (formed once on the host).
-struct RefF {
-  float rho0, Ux, Uy, Uz;
-  float c1[27];
-  float cU2[27];
+// ------------------------------------------------------- two-lane binary32
+// Two independent binary32 values in the packed FP32 instructions (one issue
+// slot for both lanes): two nodes, or the two runs of an interleaved pair.
+// Each lane rounds like the scalar operation.
+struct F2 {
+  float2 v;
 };
 
-// Equilibrium deviation of direction I from the deviations alone:
-//   g0_i = w_i [ drho (1 + e_i(U)) + (rho0 + drho) (e_i(u) - e_i(U)) ],
-//   e_i(u) - e_i(U) = 3 xi.du + 4.5 (xi.du)(2 xi.U + xi.du) - dusq + T3_i(dA),
-// with dusq = 1.5 du.(2U + du) and dA the deviations of the third-order
-// coefficients (third_coeffs).  MOV = false folds U = 0: c1 = 1, cU2 = 0,
-// and the expression is the rest-state equilibrium w_i [drho + rho e_i(u)].
-template <class L, int I, bool MOV>
-__device__ __forceinline__ float eq_i(float drho, float rho, float dux, float duy, float duz,
-                                      float dusq, const float (&dA)[7], const RefF& R) {
-  const float cdu = cdot<L, I>(dux, duy, duz);
-  const float cu2 = MOV ? R.cU2[I] : 0.0f;
-  const float c1 = MOV ? R.c1[I] : 1.0f;
-  const float de = 3.0f * cdu + 4.5f * cdu * (cu2 + cdu) - dusq + third<L, I>(dA);
-  return wmul<L, I>(drho * c1 + rho * de);
+// The arithmetic below is written once over T = float or F2 (double on the
+// host, for checks).
+template <class T>
+__host__ __device__ __forceinline__ T bc(float a) {
+  if constexpr (std::is_same<T, F2>::value)
+    return {make_float2(a, a)};
+  else
+    return T(a);
+}
+__host__ __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__host__ __device__ __forceinline__ double vfma(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
+// a - b, one instruction: b * (-1) is exact, the sum is rounded once
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+  return {__ffma2_rn(b.v, make_float2(-1.0f, -1.0f), a.v)};
+}
+// k x + y with a compile-time or warp-uniform binary32 factor
+template <class T>
+__host__ __device__ __forceinline__ T kfma(float k, T x, T y) { return vfma(bc<T>(k), x, y); }
+template <class T>
+__host__ __device__ __forceinline__ T kmul(float k, T x) { return bc<T>(k) * x; }
+
+// 1 / x for x near 1: the hardware's approximation (one ulp) and one
+// Newton-Raphson step, r + r (1 - x r).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+template <class T>
+__host__ __device__ __forceinline__ T vrcp(T x) {
+#ifdef __CUDA_ARCH__
+  T r;
+  if constexpr (std::is_same<T, F2>::value)
+    r = {make_float2(rcp_approx(x.v.x), rcp_approx(x.v.y))};
+  else
+    r = rcp_approx(x);
+  return vfma(r, vfma(bc<T>(-1.0f) * x, r, bc<T>(1.0f)), r);
+#else
+  return bc<T>(1.0f) / x;
+#endif
+}
+
+// x / N without a systematic bias: 1 / N as a binary32 head and tail (a
+// rounded constant would shift mass or momentum by the same relative amount
+// at every update, a drift that adds up over long runs).
+template <int N, class T>
+__host__ __device__ __forceinline__ T over(T x) {
+  if constexpr (std::is_same<T, double>::value) {
+    return x / N;
+  } else {
+    constexpr float hi = float(1.0 / N);
+    constexpr float lo = float(1.0 / N - double(hi));
+    return vfma(bc<T>(hi), x, kmul(lo, x));
+  }
+}
+
+// Index of direction (x, y, z).
+template <class L>
+__host__ __device__ constexpr int dir(int x, int y, int z) {
+  for (int i = 0; i < L::Q; ++i)
+    if (L::c(i, 0) == x && L::c(i, 1) == y && L::c(i, 2) == z) return i;
+  return -1;
+}
+
+// Second-order components, in this order.
+enum { XX = 0, YY, ZZ, XY, XZ, YZ };
+
+// Moments of a population set: d = sum g, j = sum xi g, P = sum xi xi g.
+// Opposite directions enter only through their sum (even moments) and
+// difference (odd ones).
+template <class L, class T>
+__host__ __device__ __forceinline__ void moments2(const T (&g)[L::Q], T& d, T (&j)[3],
+                                                  T (&P)[6]) {
+  auto even = [&](auto X, auto Y, auto Z) {
+    constexpr int x = decltype(X)::value, y = decltype(Y)::value, z = decltype(Z)::value;
+    return g[dir<L>(x, y, z)] + g[dir<L>(-x, -y, -z)];
+  };
+  auto odd = [&](auto X, auto Y, auto Z) {
+    constexpr int x = decltype(X)::value, y = decltype(Y)::value, z = decltype(Z)::value;
+    return g[dir<L>(x, y, z)] - g[dir<L>(-x, -y, -z)];
+  };
+  constexpr std::integral_constant<int, 0> o{};
+  constexpr std::integral_constant<int, 1> p{};
+  constexpr std::integral_constant<int, -1> m{};
+  const T sx = even(p, o, o), dx = odd(p, o, o), sy = even(o, p, o), dy = odd(o, p, o);
+  const T s1 = even(p, p, o), d1 = odd(p, p, o), s2 = even(p, m, o), d2 = odd(p, m, o);
+  const T sxy = s1 + s2;
+  if constexpr (L::D == 2) {
+    P[XX] = sx + sxy;
+    P[YY] = sy + sxy;
+    P[XY] = s1 - s2;
+    P[ZZ] = P[XZ] = P[YZ] = bc<T>(0.0f);
+    d = (g[0] + sx) + P[YY];
+    j[0] = dx + (d1 + d2);
+    j[1] = dy + (d1 - d2);
+    j[2] = bc<T>(0.0f);
+  } else {
+    const T sz = even(o, o, p), dz = odd(o, o, p);
+    const T s3 = even(p, o, p), d3 = odd(p, o, p), s4 = even(p, o, m), d4 = odd(p, o, m);
+    const T s5 = even(o, p, p), d5 = odd(o, p, p), s6 = even(o, p, m), d6 = odd(o, p, m);
+    const T sxz = s3 + s4, syz = s5 + s6;
+    T ax = sx, ay = sy, az = sz;
+    P[XY] = s1 - s2;
+    P[XZ] = s3 - s4;
+    P[YZ] = s5 - s6;
+    d = ((g[0] + sx) + (sy + sz)) + ((sxy + sxz) + syz);
+    j[0] = (dx + (d1 + d2)) + (d3 + d4);
+    j[1] = (dy + (d1 - d2)) + (d5 + d6);
+    j[2] = (dz + (d3 - d4)) + (d5 - d6);
+    if constexpr (L::Q == 27) {
+      // corners (1,1,1), (1,1,-1), (1,-1,1), (-1,1,1) and their opposites
+      const T c1 = even(p, p, p), e1 = odd(p, p, p), c2 = even(p, p, m), e2 = odd(p, p, m);
+      const T c3 = even(p, m, p), e3 = odd(p, m, p), c4 = even(m, p, p), e4 = odd(m, p, p);
+      const T c12 = c1 + c2, c34 = c3 + c4, b12 = c1 - c2, b34 = c3 - c4, c = c12 + c34;
+      ax = ax + c;
+      ay = ay + c;
+      az = az + c;
+      d = d + c;
+      P[XY] = P[XY] + (c12 - c34);
+      P[XZ] = P[XZ] + (b12 + b34);
+      P[YZ] = P[YZ] + (b12 - b34);
+      const T e12 = e1 + e2, e34 = e3 - e4;
+      j[0] = j[0] + (e12 + e34);
+      j[1] = j[1] + (e12 - e34);
+      j[2] = j[2] + ((e1 - e2) + (e3 + e4));
+    }
+    P[XX] = ax + (sxy + sxz);
+    P[YY] = ay + (sxy + syz);
+    P[ZZ] = az + (sxz + syz);
+  }
+}
+
+// Populations of a Hermite expansion (eq. fEqH to third order): direction i
+// of  w_i [d + 3 xi.j + 4.5 H2_i:B + T3_i(A)],  each handed to
+// emit(integral_constant<i>, value).  Takes C = A / 4 (order XXY .. XYZ).
+// The coefficients are folded with the weights, which leaves powers of two
+// and a few thirds (over<N>): a direction costs two to four operations
+// instead of a polynomial of its own.
+//   D2Q9, D3Q19: opposite directions share E +- O.  Along an axis
+//     O = j_a / 6 ... - A_bba / 2 (- A_cca / 2), on an edge
+//     (j_a / 3 + A_bba) / 4 +- (j_b / 3 + A_aab) / 4.
+//   D3Q27: the raw moments M_pqr (p, q, r <= 2) of the expansion, halved
+//     once per axis with a nonzero power, then one axis at a time
+//     g_0 = M_0 - 2 M_2, g_+- = M_2 +- M_1.
+template <class L, class T, class Emit>
+__host__ __device__ __forceinline__ void expand(T d, const T (&j)[3], const T (&B)[6],
+                                                const T (&C)[7], Emit&& emit) {
+  // the pair (x, y, z) and its opposite from the even and the odd part, k O
+  auto pair = [&](auto X, auto Y, auto Z, T even, float k, T odd) {
+    constexpr int x = decltype(X)::value, y = decltype(Y)::value, z = decltype(Z)::value;
+    emit(std::integral_constant<int, dir<L>(x, y, z)>{}, kfma(k, odd, even));
+    emit(std::integral_constant<int, dir<L>(-x, -y, -z)>{}, kfma(-k, odd, even));
+  };
+  constexpr std::integral_constant<int, 0> o{};
+  constexpr std::integral_constant<int, 1> p{};
+  constexpr std::integral_constant<int, -1> m{};
+  const T jx = over<12>(j[0]), jy = over<12>(j[1]);
+  if constexpr (L::Q == 9) {
+    const T d9 = over<9>(d), t3 = over<3>(B[XX] + B[YY]);
+    emit(std::integral_constant<int, 0>{}, kfma(-2.0f, t3, kmul(4.0f, d9)));
+    const T ax = kfma(-0.5f, t3, d9), c = kmul(0.25f, d9 + t3);
+    pair(p, o, o, kfma(0.5f, B[XX], ax), 4.0f, kfma(-0.5f, C[YYX], jx));
+    pair(o, p, o, kfma(0.5f, B[YY], ax), 4.0f, kfma(-0.5f, C[XXY], jy));
+    const T X = jx + C[YYX], Y = jy + C[XXY];
+    pair(p, p, o, kfma(0.25f, B[XY], c), 1.0f, X + Y);
+    pair(p, m, o, kfma(-0.25f, B[XY], c), 1.0f, X - Y);
+  } else if constexpr (L::Q == 19) {
+    const T jz = over<12>(j[2]);
+    const T s9 = over<9>(kfma(-1.5f, (B[XX] + B[YY]) + B[ZZ], d));
+    emit(std::integral_constant<int, 0>{}, kmul(3.0f, s9));
+    const T a = kmul(0.5f, s9), e = kmul(0.25f, s9);
+    pair(p, o, o, kfma(0.25f, B[XX], a), 2.0f, jx - (C[YYX] + C[ZZX]));
+    pair(o, p, o, kfma(0.25f, B[YY], a), 2.0f, jy - (C[XXY] + C[ZZY]));
+    pair(o, o, p, kfma(0.25f, B[ZZ], a), 2.0f, jz - (C[XXZ] + C[YYZ]));
+    auto edge = [&](auto X1, auto Y1, auto Z1, auto X2, auto Y2, auto Z2, T Baa, T Bbb, T Bab,
+                    T X, T Y) {
+      const T c = kfma(0.125f, Bbb, kfma(0.125f, Baa, e));
+      pair(X1, Y1, Z1, kfma(0.25f, Bab, c), 1.0f, X + Y);
+      pair(X2, Y2, Z2, kfma(-0.25f, Bab, c), 1.0f, X - Y);
+    };
+    edge(p, p, o, p, m, o, B[XX], B[YY], B[XY], jx + C[YYX], jy + C[XXY]);
+    edge(p, o, p, p, o, m, B[XX], B[ZZ], B[XZ], jx + C[ZZX], jz + C[XXZ]);
+    edge(o, p, p, o, p, m, B[YY], B[ZZ], B[YZ], jy + C[ZZY], jz + C[YYZ]);
+  } else {
+    const T jz = over<12>(j[2]);
+    T M[3][3][3];  // [p][q][r]
+    const T d3 = over<3>(d), d9 = over<9>(d);
+    const T qx = over<3>(B[XX]), qy = over<3>(B[YY]), qz = over<3>(B[ZZ]);
+    M[0][0][0] = d;
+    M[1][0][0] = kmul(0.5f, j[0]);
+    M[0][1][0] = kmul(0.5f, j[1]);
+    M[0][0][1] = kmul(0.5f, j[2]);
+    M[2][0][0] = kmul(0.5f, B[XX] + d3);
+    M[0][2][0] = kmul(0.5f, B[YY] + d3);
+    M[0][0][2] = kmul(0.5f, B[ZZ] + d3);
+    M[1][1][0] = kmul(0.25f, B[XY]);
+    M[1][0][1] = kmul(0.25f, B[XZ]);
+    M[0][1][1] = kmul(0.25f, B[YZ]);
+    const T qxy = (qx + qy) + d9;
+    M[2][2][0] = kmul(0.25f, qxy);
+    M[2][0][2] = kmul(0.25f, (qx + qz) + d9);
+    M[0][2][2] = kmul(0.25f, (qy + qz) + d9);
+    M[2][2][2] = over<24>(qxy + qz);
+    M[2][1][0] = C[XXY] + jy;
+    M[2][0][1] = C[XXZ] + jz;
+    M[1][2][0] = C[YYX] + jx;
+    M[0][2][1] = C[YYZ] + jz;
+    M[1][0][2] = C[ZZX] + jx;
+    M[0][1][2] = C[ZZY] + jy;
+    M[1][1][1] = kmul(0.5f, C[XYZ]);
+    M[2][2][1] = over<6>(M[2][0][1] + C[YYZ]);
+    M[2][1][2] = over<6>(M[2][1][0] + C[ZZY]);
+    M[1][2][2] = over<6>(M[1][2][0] + C[ZZX]);
+    M[2][1][1] = over<24>(B[YZ]);
+    M[1][2][1] = over<24>(B[XZ]);
+    M[1][1][2] = over<24>(B[XY]);
+    auto inv = [](T& a, T& b, T& c) {  // (M_0, M_1, M_2) -> (g_-, g_0, g_+)
+      const T m1 = b, m2 = c;
+      b = kfma(-2.0f, m2, a);
+      a = m2 - m1;
+      c = m2 + m1;
+    };
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) inv(M[0][q][r], M[1][q][r], M[2][q][r]);
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) inv(M[x][0][r], M[x][1][r], M[x][2][r]);
+    sfor<9>([&](auto K) {
+      constexpr int x = decltype(K)::value / 3, y = decltype(K)::value % 3;
+      inv(M[x][y][0], M[x][y][1], M[x][y][2]);
+      emit(std::integral_constant<int, dir<L>(x - 1, y - 1, -1)>{}, M[x][y][0]);
+      emit(std::integral_constant<int, dir<L>(x - 1, y - 1, 0)>{}, M[x][y][1]);
+      emit(std::integral_constant<int, dir<L>(x - 1, y - 1, 1)>{}, M[x][y][2]);
+    });
+  }
+}
+
+// Reference state (rho0, U) of the shifted storage in binary32, with the
+// products the deviations need, formed on the host in double precision.
+struct RefF {
+  float rho0;
+  float U[3];
+  float m[3];  // rho0 U_a
+  float k[4];  // rho0 U_a U_a / 4, and rho0 U_x U_y / 4
+};
+
+// Second- and third-order deviations of the equilibrium from the reference,
+//   dP_ab  = rho u_a u_b - rho0 U_a U_b = j_a u_b + rho0 U_a du_b,
+//   dA_aab = rho u_a u_a u_b - rho0 U_a U_a U_b = dP_aa u_b + rho0 U_a U_a du_b,
+// with j = rho u - rho0 U: no large terms cancel.  MOV = false: U = 0.
+template <class L, bool MOV, class T>
+__host__ __device__ __forceinline__ void second_dev(const T (&j)[3], const T (&u)[3],
+                                                    const T (&du)[3], const RefF& R,
+                                                    T (&dP)[6]) {
+  auto prod = [&](int a, int b) {
+    const T x = MOV ? kmul(R.m[a], du[b]) : bc<T>(0.0f);
+    return MOV ? vfma(j[a], u[b], x) : j[a] * u[b];
+  };
+  dP[XX] = prod(0, 0);
+  dP[YY] = prod(1, 1);
+  dP[XY] = prod(0, 1);
+  dP[ZZ] = dP[XZ] = dP[YZ] = bc<T>(0.0f);
+  if constexpr (L::D == 3) {
+    dP[ZZ] = prod(2, 2);
+    dP[XZ] = prod(0, 2);
+    dP[YZ] = prod(1, 2);
+  }
+}
+
+// Third-order coefficients over four, C_aab = (V_aab + 2 u_a W_ab) / 4 with
+// V_aab = Q_aa u_b + rho0 U_a U_a du_b (W_ab = 0: the equilibrium's own
+// dA / 4 for Q = dP): with Q = dP + a1, W = a1 this is
+// dA + a1^(3) of eq. a13RR, (a1^(3)_aab = 2 u_a a1_ab + u_b a1_aa).
+template <class L, bool MOV, bool W1, class T>
+__host__ __device__ __forceinline__ void third_dev(const T (&Q)[6], const T (&W)[6],
+                                                   const T (&u)[3], const T (&du)[3],
+                                                   const RefF& R, T (&C)[7]) {
+  T uq[3], uh[3];
+#pragma unroll
+  for (int a = 0; a < L::D; ++a) {
+    uq[a] = kmul(0.25f, u[a]);
+    uh[a] = kmul(0.5f, u[a]);
+  }
+  auto aab = [&](int a, int b, int aa, int ab) {
+    T c = bc<T>(0.0f);
+    if constexpr (MOV) c = kmul(R.k[a], du[b]);
+    if constexpr (W1) c = MOV ? vfma(uh[a], W[ab], c) : uh[a] * W[ab];
+    return (MOV || W1) ? vfma(uq[b], Q[aa], c) : uq[b] * Q[aa];
+  };
+  C[XXY] = aab(0, 1, XX, XY);
+  C[YYX] = aab(1, 0, YY, XY);
+  if constexpr (L::D == 3) {
+    C[XXZ] = aab(0, 2, XX, XZ);
+    C[YYZ] = aab(1, 2, YY, YZ);
+    C[ZZX] = aab(2, 0, ZZ, XZ);
+    C[ZZY] = aab(2, 1, ZZ, YZ);
+    if constexpr (L::Q == 27) {
+      T c = bc<T>(0.0f);
+      if constexpr (MOV) c = kmul(R.k[3], du[2]);
+      if constexpr (W1) {
+        c = MOV ? vfma(uq[0], W[YZ], c) : uq[0] * W[YZ];
+        c = vfma(uq[1], W[XZ], c);
+      }
+      C[XYZ] = (MOV || W1) ? vfma(uq[2], Q[XY], c) : uq[2] * Q[XY];
+    }
+  }
+}
+
+// Equilibrium deviations f0(rho0 + drho, U + du) - f0(rho0, U), direction by
+// direction to emit(integral_constant<i>, value).
+template <class L, class Emit>
+__host__ __device__ __forceinline__ void equilibrium_emit(float drho, float dux, float duy,
+                                                          float duz, const RefF& R, Emit&& emit) {
+  const float du[3] = {dux, duy, L::D == 3 ? duz : 0.0f};
+  float u[3], j[3], dP[6], C[7];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    u[a] = R.U[a] + du[a];
+    j[a] = fmaf(drho, u[a], R.rho0 * du[a]);
+  }
+  second_dev<L, true>(j, u, du, R, dP);
+  third_dev<L, true, false>(dP, dP, u, du, R, C);
+  expand<L>(drho, j, dP, C, emit);
 }
 
 // All q equilibrium deviations (binary32) at (rho0 + drho, U + du).
 template <class L>
-__device__ __forceinline__ void equilibrium_f(float drho, float dux, float duy, float duz,
-                                              const RefF& R, float (&g0)[L::Q]) {
-  const float Ux = R.Ux, Uy = R.Uy, Uz = (L::D == 3) ? R.Uz : 0.0f;
-  if constexpr (L::D == 2) duz = 0.0f;
-  const float ux = Ux + dux, uy = Uy + duy, uz = Uz + duz;
-  float A[7], dA[7];
-  third_coeffs(ux, uy, uz, dux, duy, duz, Ux, Uy, Uz, A, dA);
-  const float dusq = 1.5f * (dux * (ux + Ux) + duy * (uy + Uy) + duz * (uz + Uz));
-  const float rho = R.rho0 + drho;
-  sfor<L::Q>([&](auto I) {
-    constexpr int i = decltype(I)::value;
-    g0[i] = eq_i<L, i, true>(drho, rho, dux, duy, duz, dusq, dA, R);
-  });
+__host__ __device__ __forceinline__ void equilibrium_f(float drho, float dux, float duy, float duz,
+                                                       const RefF& R, float (&g0)[L::Q]) {
+  equilibrium_emit<L>(drho, dux, duy, duz, R,
+                      [&](auto I, float v) { g0[decltype(I)::value] = v; });
 }
 
 // Density and velocity deviations of shifted populations:
@@ -342,18 +603,19 @@ __device__ __forceinline__ void deviations(const float (&g)[L::Q], const RefF& R
                                            float& dux, float& duy, float& duz) {
   float jx, jy, jz;
   moments<L>(g, drho, jx, jy, jz);
-  const float inv = 1.0f / (R.rho0 + drho);
-  dux = (jx - drho * R.Ux) * inv;
-  duy = (jy - drho * R.Uy) * inv;
-  duz = (L::D == 3) ? (jz - drho * R.Uz) * inv : 0.0f;
+  const float inv = vrcp(R.rho0 + drho);
+  dux = (jx - drho * R.U[0]) * inv;
+  duy = (jy - drho * R.U[1]) * inv;
+  duz = (L::D == 3) ? (jz - drho * R.U[2]) * inv : 0.0f;
 }
 
 // Strain-rate input of the hybrid collision (eq. a1ij_HRR):
 // a1 <- sig a1 + ks rho S with ks = -2 tau cs^2 (1 - sig);
 // s = (S_xx, S_yy, S_zz, S_xy, S_xz, S_yz).
+template <class T>
 struct HrrIn {
   float sig, ks;
-  float s[6];
+  T s[6];
 };
 
 // Collision of shifted populations; the post-collision value of each
@@ -364,127 +626,63 @@ struct HrrIn {
 // needs hy).  omega = 1 - 1/tau.
 // MOV = false: the reference velocity is zero (rest-state shift) and every
 // term in U is folded away at compile time.
-template <class L, int COLL, bool MOV, class Emit>
-__device__ __forceinline__ void collide_emit(const float (&g)[L::Q], float omega, const RefF& Rin,
-                                             Emit&& emit, const HrrIn* hy = nullptr) {
-  // (moments, deviations and the equilibrium of each direction)
-  const float Ux = MOV ? Rin.Ux : 0.0f, Uy = MOV ? Rin.Uy : 0.0f,
-              Uz = (MOV && L::D == 3) ? Rin.Uz : 0.0f, rho0 = Rin.rho0;
-  float drho, jv[3], pd[3], po[3];
-  moments2<L>(g, drho, jv, pd, po);
-  const float jx = jv[0], jy = jv[1], jz = jv[2];
-  const float rho = rho0 + drho;
-  const float inv = __frcp_rn(rho);  // correctly rounded, as 1.0f / rho
-  const float dux = (jx - drho * Ux) * inv, duy = (jy - drho * Uy) * inv,
-              duz = (L::D == 3) ? (jz - drho * Uz) * inv : 0.0f;
-  const float ux = Ux + dux, uy = Uy + duy, uz = Uz + duz;
-  float Ae[7], dAe[7];
-  third_coeffs(ux, uy, uz, dux, duy, duz, Ux, Uy, Uz, Ae, dAe);
-  const float dusq = 1.5f * (dux * (ux + Ux) + duy * (uy + Uy) + duz * (uz + Uz));
-  // Opposite directions share the even part of the equilibrium deviation
-  // and of f^(1) and differ in the sign of the odd part:
-  //   de_i = Ev + Od, de_opp(i) = Ev - Od,
-  //   Ev = 4.5 (xi.du)(2 xi.U + xi.du) - dusq,  Od = 3 xi.du + T3_i(dA).
-  // X_i such that g0_i = w_i X_i
-  auto eq_pair = [&](auto I, float& xi, float& xj) {
-    constexpr int i = decltype(I)::value;
-    constexpr int j = opp<L>(i);
-    const float cdu = cdot<L, i>(dux, duy, duz);
-    const float cu2 = MOV ? Rin.cU2[i] : 0.0f;
-    const float ev = 4.5f * cdu * (cu2 + cdu) - dusq;
-    const float od = 3.0f * cdu + third<L, i>(dAe);
-    const float c1i = MOV ? Rin.c1[i] : 1.0f, c1j = MOV ? Rin.c1[j] : 1.0f;
-    xi = drho * c1i + rho * (ev + od);
-    xj = drho * c1j + rho * (ev - od);
-  };
-  const float x00 = drho * (MOV ? Rin.c1[0] : 1.0f) - rho * dusq;  // rest direction
-  constexpr int NP = (L::Q - 1) / 2;
+// The regularized post-collision state f0 + omega f1 is one Hermite
+// expansion in d, j (both conserved), B = dP + omega a1 and
+// A = dA + omega a1^(3), so equilibrium and off-equilibrium parts are added
+// as moments and expanded into populations once -- the updates in binary16
+// storage are bound by these instructions, not by HBM (a polynomial per
+// direction for each part, with the zero coefficients multiplied out, took
+// 445 us for the fine update of a binary16 D3Q19 slab of 16.4 M nodes, this
+// form 355; paired D2Q9 runs 80.6 -> 65.9 us for 33 x 513^2 nodes; in
+// binary32 D3Q19 5.48 -> 5.77 TB/s, D2Q9 5.69 -> 5.88 TB/s).
+template <class L, int COLL, bool MOV, class T, class Emit>
+__host__ __device__ __forceinline__ void collide_emit(const T (&g)[L::Q], float omega,
+                                                      const RefF& R, Emit&& emit,
+                                                      const HrrIn<T>* hy = nullptr) {
+  T d, j[3], P[6], dP[6], C[7], u[3], du[3];
+  moments2<L>(g, d, j, P);
+  const T rho = bc<T>(R.rho0) + d, inv = vrcp(rho);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (a >= L::D) {
+      u[a] = du[a] = bc<T>(0.0f);
+    } else if constexpr (MOV) {
+      du[a] = kfma(-R.U[a], d, j[a]) * inv;
+      u[a] = bc<T>(R.U[a]) + du[a];
+    } else {
+      u[a] = du[a] = j[a] * inv;
+    }
+  }
+  second_dev<L, MOV>(j, u, du, R, dP);
   if constexpr (COLL == 0) {
-    const float g00 = wmul<L, 0>(x00);
-    emit(std::integral_constant<int, 0>{}, g00 + omega * (g[0] - g00));
-    sfor<NP>([&](auto P) {
-      constexpr int i = pair_first<L>(decltype(P)::value);
-      constexpr int j = opp<L>(i);
-      float xi, xj;
-      eq_pair(std::integral_constant<int, i>{}, xi, xj);
-      const float gi = wmul<L, i>(xi), gj = wmul<L, j>(xj);
-      emit(std::integral_constant<int, i>{}, gi + omega * (g[i] - gi));
-      emit(std::integral_constant<int, j>{}, gj + omega * (g[j] - gj));
+    third_dev<L, MOV, false>(dP, dP, u, du, R, C);
+    expand<L>(d, j, dP, C, [&](auto I, T v) {
+      emit(I, kfma(omega, g[decltype(I)::value] - v, v));
     });
   } else {
-    // second moments of the deviations g
-    const float pxx = pd[0], pyy = pd[1], pzz = pd[2], pxy = po[0], pxz = po[1], pyz = po[2];
-    // a1 = sum xi xi g - drho cs^2 I - drho u u - rho0 (u u - U U),
-    // with u_a u_b - U_a U_b = du_a u_b + U_a du_b
-    const float dc = drho * (1.0f / 3.0f);
-    float axx, ayy, azz, axy, axz, ayz;
-    if constexpr (MOV) {
-      axx = pxx - dc - drho * ux * ux - rho0 * dux * (ux + Ux);
-      ayy = pyy - dc - drho * uy * uy - rho0 * duy * (uy + Uy);
-      azz = (L::D == 3) ? pzz - dc - drho * uz * uz - rho0 * duz * (uz + Uz) : 0.0f;
-      axy = pxy - drho * ux * uy - rho0 * (dux * uy + Ux * duy);
-      axz = (L::D == 3) ? pxz - drho * ux * uz - rho0 * (dux * uz + Ux * duz) : 0.0f;
-      ayz = (L::D == 3) ? pyz - drho * uy * uz - rho0 * (duy * uz + Uy * duz) : 0.0f;
-    } else {  // U = 0
-      axx = pxx - rho * ux * ux - dc;
-      ayy = pyy - rho * uy * uy - dc;
-      azz = (L::D == 3) ? pzz - rho * uz * uz - dc : 0.0f;
-      axy = pxy - rho * ux * uy;
-      axz = (L::D == 3) ? pxz - rho * ux * uz : 0.0f;
-      ayz = (L::D == 3) ? pyz - rho * uy * uz : 0.0f;
-    }
-    if constexpr (COLL == 3) {
-      const float kr = hy->ks * rho;
-      axx = hy->sig * axx + kr * hy->s[0];
-      ayy = hy->sig * ayy + kr * hy->s[1];
-      axy = hy->sig * axy + kr * hy->s[3];
-      if constexpr (L::D == 3) {
-        azz = hy->sig * azz + kr * hy->s[2];
-        axz = hy->sig * axz + kr * hy->s[4];
-        ayz = hy->sig * ayz + kr * hy->s[5];
-      }
-    }
-    float A[7] = {0, 0, 0, 0, 0, 0, 0};
-    if constexpr (COLL >= 2) {
-      A[XXY] = 2.0f * ux * axy + uy * axx;
-      A[YYX] = 2.0f * uy * axy + ux * ayy;
-      if constexpr (L::D == 3) {
-        A[XXZ] = 2.0f * ux * axz + uz * axx;
-        A[YYZ] = 2.0f * uy * ayz + uz * ayy;
-        A[ZZX] = 2.0f * uz * axz + ux * azz;
-        A[ZZY] = 2.0f * uz * ayz + uy * azz;
-        A[XYZ] = ux * ayz + uy * axz + uz * axy;
-      }
-    }
-    // f^(1): 4.5 H2:a1 is even in xi (shared by a pair), T3(a1^(3)) is odd
-    auto h2a_of = [&](auto I) {
-      constexpr int i = decltype(I)::value;
-      constexpr int cx = L::c(i, 0), cy = L::c(i, 1), cz = L::c(i, 2);
-      constexpr float dxx = float(4.5 * (double(cx * cx) - 1.0 / 3.0));
-      constexpr float dyy = float(4.5 * (double(cy * cy) - 1.0 / 3.0));
-      constexpr float oxy = 9.0f * float(cx * cy);
-      float h = dxx * axx + dyy * ayy + oxy * axy;
-      if constexpr (L::D == 3) {
-        constexpr float dzz = float(4.5 * (double(cz * cz) - 1.0 / 3.0));
-        constexpr float oxz = 9.0f * float(cx * cz), oyz = 9.0f * float(cy * cz);
-        h += dzz * azz + oxz * axz + oyz * ayz;
-      }
-      return h;
+    // omega a1, a1_ab = P_ab - d cs^2 delta_ab - dP_ab
+    const T d3 = over<3>(d);
+    T a1[6], B[6];
+    auto fill = [&](int k) {
+      T x = (k < 3 ? P[k] - d3 : P[k]) - dP[k];
+      if constexpr (COLL == 3) x = vfma(kmul(hy->ks, rho), hy->s[k], kmul(hy->sig, x));
+      a1[k] = kmul(omega, x);
+      B[k] = dP[k] + a1[k];
     };
-    // post_i = w_i (X_i + omega F_i) with F_i = 4.5 H2_i:a1 + T3_i(a1^(3))
-    emit(std::integral_constant<int, 0>{},
-         wmul<L, 0>(x00 + omega * h2a_of(std::integral_constant<int, 0>{})));
-    sfor<NP>([&](auto P) {
-      constexpr int i = pair_first<L>(decltype(P)::value);
-      constexpr int j = opp<L>(i);
-      float xi, xj;
-      eq_pair(std::integral_constant<int, i>{}, xi, xj);
-      const float h = h2a_of(std::integral_constant<int, i>{});
-      float t = 0.0f;
-      if constexpr (COLL >= 2) t = third<L, i>(A);
-      emit(std::integral_constant<int, i>{}, wmul<L, i>(xi + omega * (h + t)));
-      emit(std::integral_constant<int, j>{}, wmul<L, j>(xj + omega * (h - t)));
-    });
+    fill(XX);
+    fill(YY);
+    fill(XY);
+    a1[ZZ] = a1[XZ] = a1[YZ] = B[ZZ] = B[XZ] = B[YZ] = bc<T>(0.0f);
+    if constexpr (L::D == 3) {
+      fill(ZZ);
+      fill(XZ);
+      fill(YZ);
+    }
+    if constexpr (COLL == 1)
+      third_dev<L, MOV, false>(dP, a1, u, du, R, C);
+    else
+      third_dev<L, MOV, true>(B, a1, u, du, R, C);
+    expand<L>(d, j, B, C, emit);
   }
 }
 

@@ -11,25 +11,18 @@ namespace detail {
 
 inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// binary32 reference state with the per-direction constants 1 + e_i(U) and
-// 2 xi_i.U, formed in double precision.
+// binary32 reference state and its products, formed in double precision.
 template <class L>
 RefF make_ref_f(const RefState& r) {
+  const double U[3] = {r.U[0], r.U[1], L::D == 3 ? r.U[2] : 0.0};
   RefF R{};
   R.rho0 = (float)r.rho0;
-  R.Ux = (float)r.U[0];
-  R.Uy = (float)r.U[1];
-  R.Uz = L::D == 3 ? (float)r.U[2] : 0.0f;
-  const double Uz = L::D == 3 ? r.U[2] : 0.0;
-  double eU[L::Q];
-  // e_i(U) = (f0_i(1, U) - w_i) / w_i
-  double f0[L::Q];
-  equilibrium_dev<L, double>(0.0, r.U[0], r.U[1], Uz, 1.0, 0.0, 0.0, 0.0, f0);
-  for (int i = 0; i < L::Q; ++i) {
-    eU[i] = f0[i] / L::w(i);
-    R.c1[i] = (float)(1.0 + eU[i]);
-    R.cU2[i] = (float)(2.0 * (L::c(i, 0) * r.U[0] + L::c(i, 1) * r.U[1] + L::c(i, 2) * Uz));
+  for (int a = 0; a < 3; ++a) {
+    R.U[a] = (float)U[a];
+    R.m[a] = (float)(r.rho0 * U[a]);
+    R.k[a] = (float)(0.25 * r.rho0 * U[a] * U[a]);
   }
+  R.k[3] = (float)(0.25 * r.rho0 * U[0] * U[1]);
   return R;
 }
 
