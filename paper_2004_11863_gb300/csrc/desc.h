@@ -158,6 +158,36 @@ struct TnDesc {
   int boxed[3];
 };
 
+// Time interpolation of a capture (eq. TempInt; see capture_item).
+struct TimeInt {
+  int on;
+  int s_m1, s_0;  // slots holding t - 1 (replaced) and t
+  float w0, w1, w2;
+};
+
+// Special nodes of a 2D level update, rebuilt and collided by blocks of their
+// own in the update's launch (kernels_edge.cuh).  Up to four faces.
+struct Edge2d {
+  int nz;        // leading z-slices of the grid that hold these blocks (0: none)
+  int wide;      // several lanes per node
+  int nb, nt;    // rebuilt outer nodes and TN nodes per run (0: the update's own blocks
+                 // take them like any other node)
+  int nf;        // faces of the level's own box
+  int b_start[5], b_axis[4], b_side[4], b_lo[4];  // outer nodes by face, along its tangent
+  int r_start[4];       // history-ring offset of each face
+  int p_boxed[2], p_n[2];  // parent geometry along each axis
+  const float* hist;    // the slot to read, run 0
+  long long K, run_stride;  // ring entries; floats between runs
+  float resc;           // eq. rescff
+  int tf;        // faces of the child's box
+  int t_start[5], t_axis[4], t_ra[4], t_lo[4];  // TN nodes by face: normal and first tangent
+                                                // coordinate, relative to the child's box
+  int t_org[2], t_boxed[2];  // the child box's origin; axes it bounds
+  LevelView child;
+  int cpar;             // parity of the child's next update
+  float t_resc;         // eq. rescfc
+};
+
 // Persistent fused step (kernels_fused.cuh): the recorded program, the
 // launch arguments and the host-side description of the tables it reads.
 constexpr int kFusedLevels = 4;

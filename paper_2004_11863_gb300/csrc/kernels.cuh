@@ -132,6 +132,20 @@ __device__ __forceinline__ void load_post(const S* f, long long plane, const Nod
   });
 }
 
+// (drho, du, f^(1)) of a population set (deviations from the reference).
+template <class L>
+__device__ __forceinline__ void split_neq(const float (&g)[L::Q], const RefF& R, float& drho,
+                                          float& dux, float& duy, float& duz,
+                                          float (&f1)[L::Q]) {
+  deviations<L>(g, R, drho, dux, duy, duz);
+  equilibrium_emit<L>(drho, dux, duy, duz, R, [&](auto I, float g0) {
+    constexpr int i = decltype(I)::value;
+    f1[i] = g[i] - g0;
+  });
+}
+
+#include "kernels_edge.cuh"
+
 // ------------------------------------------------------- K1: level update
 // One thread per node; a warp covers 32 consecutive x of one row.
 // Launch shape of the level update per lattice and storage type: NPT nodes
@@ -288,11 +302,13 @@ template <class L, int COLL, class S, int PAR, bool MOV>
 __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
                                            : (PAR == 0 ? K1Tune<L, S>::MINB_EVEN
                                                        : K1Tune<L, S>::MINB))
-    k_stream_collide(LevelView v, float omega, RefF R, const S* __restrict__ xf) {
+    k_stream_collide(LevelView v, float omega, RefF R, const S* __restrict__ xf,
+                     const __grid_constant__ EdgeArg<L> E) {
   constexpr int NPT = K1Tune<L, S>::NPT;
+  if (edge_block<L, S, COLL, PAR, MOV>(v, omega, R, E)) return;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * NPT;
-  int z = blockIdx.z, run = 0;
+  int z = blockIdx.z - edge_slices(E), run = 0;
   if (v.batch > 1) {
     run = z / v.n[2];
     z -= run * v.n[2];
@@ -329,7 +345,7 @@ __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
   float g[NPT][L::Q];
 #pragma unroll
   for (int k = 0; k < NPT; ++k) {
-    ok[k] = (y0 + k < v.n[1]) && !inactive(v, x, y0 + k, z);
+    ok[k] = (y0 + k < v.n[1]) && !inactive(v, x, y0 + k, z) && !edge_node(v, E, x, y0 + k);
     if (ok[k]) {
       sfor<L::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -500,9 +516,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 template <class L, class S, int COLL, int PAR, bool MOV>
 __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float omega,
                                                        const RefF& R, const S* __restrict__ xf,
-                                                       int x, int y0, int z, int run) {
-  const bool ok0 = y0 < v.n[1] && !inactive(v, x, y0, z);
-  const bool ok1 = y0 + 1 < v.n[1] && !inactive(v, x, y0 + 1, z);
+                                                       const EdgeArg<L>& E, int x, int y0, int z,
+                                                       int run) {
+  const bool ok0 = y0 < v.n[1] && !inactive(v, x, y0, z) && !edge_node(v, E, x, y0);
+  const bool ok1 = y0 + 1 < v.n[1] && !inactive(v, x, y0 + 1, z) && !edge_node(v, E, x, y0 + 1);
   if (!ok0 && !ok1) return;
   S* f = static_cast<S*>(v.f) + run * v.run_stride;  // es = 1 for this kernel
   // each lane's node; an idle lane reads its partner's
@@ -561,19 +578,21 @@ template <class L, class S, int COLL, int PAR, bool MOV>
 __global__ void __launch_bounds__(128, std::is_same<S, float>::value
                                            ? (PAR ? K1X2Tune<L>::MINB1 : K1X2Tune<L>::MINB)
                                            : (PAR ? K1X2Tune<L>::MINB1_H : K1X2Tune<L>::MINB_H))
-    k_stream_collide_x2(LevelView v, float omega, RefF R, const S* __restrict__ xf) {
+    k_stream_collide_x2(LevelView v, float omega, RefF R, const S* __restrict__ xf,
+                        const __grid_constant__ EdgeArg<L> E) {
   constexpr int PZ = K1X2Pfz<S>::PZ;
+  if (edge_block<L, S, COLL, PAR, MOV>(v, omega, R, E)) return;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * 2;
   const int nzb = (v.n[2] + PZ - 1) / PZ;  // z blocks per run
-  int zc = blockIdx.z, run = 0;
+  int zc = blockIdx.z - edge_slices(E), run = 0;
   if (v.batch > 1) {
     run = zc / nzb;
     zc -= run * nzb;
   }
   if (x >= v.n[0]) return;
   if constexpr (PZ == 1) {
-    stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, x, y0, zc, run);
+    stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, E, x, y0, zc, run);
   } else {
     const S* f = static_cast<const S*>(v.f) + run * v.run_stride;
     const int ya = y0 < v.n[1] ? y0 : v.n[1] - 1, yb = y0 + 1 < v.n[1] ? y0 + 1 : ya;
@@ -599,7 +618,7 @@ __global__ void __launch_bounds__(128, std::is_same<S, float>::value
           }
         });
       }
-      stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, x, y0, z, run);
+      stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, E, x, y0, z, run);
     }
   }
 }
@@ -637,16 +656,18 @@ struct K1PairTune<D3Q27> {
 
 template <class L, int COLL, int PAR, bool MOV>
 __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
-    k_stream_collide_pair(LevelView v, float omega, RefF R, const __half* __restrict__ xf) {
+    k_stream_collide_pair(LevelView v, float omega, RefF R, const __half* __restrict__ xf,
+                          const __grid_constant__ EdgeArg<L> E) {
+  if (edge_block<L, __half, COLL, PAR, MOV>(v, omega, R, E)) return;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int npairs = (v.batch + 1) / 2;
-  int z = blockIdx.z, pair = 0;
+  int z = blockIdx.z - edge_slices(E), pair = 0;
   if (npairs > 1) {
     pair = z / v.n[2];
     z -= pair * v.n[2];
   }
-  if (x >= v.n[0] || y >= v.n[1] || inactive(v, x, y, z)) return;
+  if (x >= v.n[0] || y >= v.n[1] || inactive(v, x, y, z) || edge_node(v, E, x, y)) return;
   // half2 units: a plane is plane / 2 of them, node e sits at e
   __half2* f = reinterpret_cast<__half2*>(static_cast<__half*>(v.f) + pair * v.run_stride);
   const long long ph = v.plane / 2;
@@ -686,22 +707,26 @@ __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
   });
 }
 
-// (drho, du, f^(1)) of a population set (deviations from the reference).
-template <class L>
-__device__ __forceinline__ void split_neq(const float (&g)[L::Q], const RefF& R, float& drho,
-                                          float& dux, float& duy, float& duz,
-                                          float (&f1)[L::Q]) {
-  deviations<L>(g, R, drho, dux, duy, duz);
-  equilibrium_emit<L>(drho, dux, duy, duz, R, [&](auto I, float g0) {
-    constexpr int i = decltype(I)::value;
-    f1[i] = g[i] - g0;
-  });
-}
-
 __device__ __forceinline__ int ring_face(const long long* start, int nf, long long k) {
   int f = 0;
   while (f + 1 < nf && k >= start[f + 1]) ++f;
   return f;
+}
+
+// Parent node of history-ring entry k (32-bit division: a ring is a surface
+// of a level of fewer than 2^31 nodes; a face reaches at most one cell past
+// the parent's periodic seam).
+__device__ __forceinline__ void ring_node(const RingDesc& R, long long k, int (&P)[3]) {
+  const int fc = ring_face(R.start, R.nf, k);
+  unsigned loc = (unsigned)(k - R.start[fc]);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const unsigned e = (unsigned)R.ext[fc][a], q = loc / e;
+    int c = R.base[fc][a] + (int)(loc - q * e);
+    loc = q;
+    if (R.pper[a]) c = wrapi(c, R.pn[a]);
+    P[a] = c;
+  }
 }
 
 // ------------------------------------------------------------ K2: capture
@@ -710,21 +735,30 @@ __device__ __forceinline__ int ring_face(const long long* start, int nf, long lo
 // for an update of parity `par` into slot `s_new`.  mode 1 (set-up): store
 // (drho, du, 0) of the parent's current state (laid out after an update of
 // parity `par`) into slots `s_new` and `s_also`.
+// interpolate (eq. TempInt): the state at the child's first sub-step,
+// w0 (t - 1) + w1 t + w2 (t + 1), replaces the state at t - 1 in slot s_m1 --
+// nothing needs t - 1 after it, and the next capture overwrites that slot --
+// so each rebuild reads one slot, and every ring node is interpolated once
+// instead of once per child node whose stencil holds it.
 template <class L, class S>
 __device__ __forceinline__ void capture_item(const LevelView& p, const RingDesc& R, int par,
                                              int mode, int s_new, int s_also, const RefF& ref,
-                                             long long k, int run) {
-  const int fc = ring_face(R.start, R.nf, k);
-  long long loc = k - R.start[fc];
+                                             long long k, int run, const TimeInt& ti) {
   int P[3];
+  ring_node(R, k, P);
+  const int nv = R.nv;
+  float* h = R.hist + (long long)run * 3 * nv * R.K;
+  // the older states first: their loads fly beside the populations' (behind
+  // the stores below they could not be moved up: the slots may alias)
+  float im[4 + L::Q] = {};
+  float* hm = h + (long long)ti.s_m1 * nv * R.K + k;
+  if (ti.on) {
+    const float* h0 = h + (long long)ti.s_0 * nv * R.K + k;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int e = R.ext[fc][a];
-    int i = (int)(loc % e);
-    loc /= e;
-    int c = R.base[fc][a] + i;
-    if (R.pper[a]) c = ((c % R.pn[a]) + R.pn[a]) % R.pn[a];
-    P[a] = c;
+    for (int vv = 0; vv < 4 + L::Q; ++vv) im[vv] = ti.w1 * h0[(long long)vv * R.K];
+    if (ti.w0 != 0.0f)  // (the first step has no t - 1)
+#pragma unroll
+      for (int vv = 0; vv < 4 + L::Q; ++vv) im[vv] += ti.w0 * hm[(long long)vv * R.K];
   }
   const S* f = run_cptr<S>(p, run);
   const NodeAddr a = node_addr<L>(p, P[0], P[1], P[2]);
@@ -735,9 +769,15 @@ __device__ __forceinline__ void capture_item(const LevelView& p, const RingDesc&
     load_post<L, S>(f, p.plane, a, par, p.es, g);
   float drho, dux, duy, duz, f1[L::Q];
   split_neq<L>(g, ref, drho, dux, duy, duz, f1);
-  const int nv = R.nv;
-  float* h = R.hist + (long long)run * 3 * nv * R.K;
   const float m4[4] = {drho, dux, duy, duz};
+  if (ti.on) {
+#pragma unroll
+    for (int vv = 0; vv < 4; ++vv) hm[(long long)vv * R.K] = im[vv] + ti.w2 * m4[vv];
+    sfor<L::Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      hm[(long long)(4 + i) * R.K] = im[4 + i] + ti.w2 * f1[i];
+    });
+  }
   for (int rep = 0; rep < (mode == 0 ? 1 : 2); ++rep) {
     float* hs = h + (long long)(rep == 0 ? s_new : s_also) * nv * R.K + k;
 #pragma unroll
@@ -750,21 +790,22 @@ __device__ __forceinline__ void capture_item(const LevelView& p, const RingDesc&
 }
 
 template <class L, class S>
-__global__ void k_capture(LevelView p, RingDesc R, int par, int mode, int s_new, int s_also,
-                          RefF ref) {
+__global__ void k_capture(LevelView p, const __grid_constant__ RingDesc R, int par, int mode,
+                          int s_new, int s_also, TimeInt ti, RefF ref) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= R.K) return;
-  capture_item<L, S>(p, R, par, mode, s_new, s_also, ref, k, blockIdx.y);
+  capture_item<L, S>(p, R, par, mode, s_new, s_also, ref, k, blockIdx.y, ti);
 }
 
 // ------------------------------------------------------------- K3: inject
-// Child TF / IE nodes (the outer node layer of the child box).  wt: temporal
-// weights on the history slots s_m1, s_0, s_p1 holding t-1, t, t+1;
+// Child TF / IE nodes (the outer node layer of the child box).  slot: the
+// history slot holding the parent state at this sub-step (interpolated in
+// time by the capture on the first one, t + 1 itself on the second);
 // resc = tau_f / (2 tau_c) (eq. rescff); par: the child's next update.
 // Organised by face tiles: a block covers TI x TJ child nodes of one face of
-// the child box with G thread groups.  It first stages the temporally
-// interpolated parent history (eq. TempInt) of the parent nodes the tile's
-// stencils reach in shared memory (all threads); then the G threads of a
+// the child box with G thread groups.  It first stages the parent
+// state of the parent nodes the tile's stencils reach in shared memory (all
+// threads); then the G threads of a
 // node share its spatial stencil (eq. spaceInt, tensor product on face
 // centres), each for every G-th interpolated value; then they share its
 // rebuild (eq. rescff) and stores, each for every G-th direction.  Each
@@ -834,8 +875,7 @@ __device__ __forceinline__ void inject_rebuild(const LevelView& c, int run, int 
 
 template <class L, class S>
 __global__ void __launch_bounds__(InjTile<L>::NT)
-    k_inject(LevelView c, InjDesc J, RingDesc R, float w0, float w1, float w2, int s_m1,
-             int s_0, int s_p1, float resc, int par, RefF ref, S* xf) {
+    k_inject(LevelView c, InjDesc J, RingDesc R, int slot, float resc, int par, RefF ref, S* xf) {
   using T = InjTile<L>;
   constexpr bool SPLIT = T::G > 1;  // a node's values shared through shared memory
   __shared__ float sv[T::NV][T::WJ][T::WI];
@@ -857,10 +897,9 @@ __global__ void __launch_bounds__(InjTile<L>::NT)
   const int bx1 = pick(R.boxed, t1), bx2 = pick(R.boxed, t2);
   const int e1 = pick(R.ext[f], t1), e2 = pick(R.ext[f], t2);
   const int pn1 = pick(R.pn, t1), pn2 = pick(R.pn, t2);
-  const float* h = R.hist + (long long)run * 3 * R.nv * R.K;
-  const long long K = R.K, nv = R.nv;
-  const bool one_slot = w0 == 0.0f && w1 == 0.0f;  // uniform over the grid
-  // stage: parent window x values, interpolated in time
+  const long long K = R.K;
+  const float* h = R.hist + ((long long)run * 3 + slot) * R.nv * K;
+  // stage: parent window x values
   const int tid = (threadIdx.z * T::TJ + threadIdx.y) * T::TI + threadIdx.x;
 #pragma unroll 4
   for (int e = tid; e < T::NV * T::WJ * T::WI; e += T::NT) {
@@ -885,16 +924,7 @@ __global__ void __launch_bounds__(InjTile<L>::NT)
         idx += (long long)rj * st2;
       }
     }
-    float val = 0.0f;
-    if (ok) {
-      if (one_slot)  // the synchronous sub-step: t+1 only
-        val = w2 * h[((long long)s_p1 * nv + vv) * K + idx];
-      else
-        val = w0 * h[((long long)s_m1 * nv + vv) * K + idx] +
-              w1 * h[((long long)s_0 * nv + vv) * K + idx] +
-              w2 * h[((long long)s_p1 * nv + vv) * K + idx];
-    }
-    sv[vv][pj][pi] = val;
+    sv[vv][pj][pi] = ok ? h[vv * K + idx] : 0.0f;
   }
   __syncthreads();
   const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
@@ -947,7 +977,7 @@ __global__ void __launch_bounds__(InjTile<L>::NT)
 }
 
 // 3D rebuild with the tensor-product stencil of eq. spaceInt applied one
-// axis at a time: the block stages the temporally interpolated parent window
+// axis at a time: the block stages the parent window
 // (TI / 2 + 3 by TJ / 2 + 3 parent nodes: exactly what the tile's stencils
 // reach), interpolates it along t1 for every window row into shared memory
 // (every thread the same four taps, even child positions weighting their
@@ -968,11 +998,11 @@ struct InjSep {
 template <class L, class S>
 __global__ void __launch_bounds__(InjSep<L>::NT)
     k_inject_sep(LevelView c, const __grid_constant__ InjDesc J,
-                 const __grid_constant__ RingDesc R, float w0, float w1, float w2, int s_m1,
-                 int s_0, int s_p1, float resc, int par, RefF ref, S* xf) {
+                 const __grid_constant__ RingDesc R, int slot, float resc, int par, RefF ref,
+                 S* xf) {
   static_assert(L::D == 3, "k_inject_sep is the 3D rebuild");
   using T = InjSep<L>;
-  __shared__ float sv[T::NV][T::WJ][T::WI];  // parent window, interpolated in time
+  __shared__ float sv[T::NV][T::WJ][T::WI];  // parent window
   __shared__ float ta[T::NV][T::WJ][T::TI];  // ... and along t1
   const int run = blockIdx.y;
   int f = 0;
@@ -989,11 +1019,10 @@ __global__ void __launch_bounds__(InjSep<L>::NT)
   const int bx1 = pick(R.boxed, t1), bx2 = pick(R.boxed, t2);
   const int e1 = pick(R.ext[f], t1), e2 = pick(R.ext[f], t2);
   const int pn1 = pick(R.pn, t1), pn2 = pick(R.pn, t2);
-  const float* h = R.hist + (long long)run * 3 * R.nv * R.K;
-  const long long K = R.K, nv = R.nv;
-  const bool one_slot = w0 == 0.0f && w1 == 0.0f;  // uniform over the grid
+  const long long K = R.K;
+  const float* h = R.hist + ((long long)run * 3 + slot) * R.nv * K;
   const int tid = threadIdx.y * T::TI + threadIdx.x;
-  // stage (eq. TempInt)
+  // stage
 #pragma unroll(T::UNR)
   for (int e = tid; e < T::NV * T::WJ * T::WI; e += T::NT) {
     const int pi = e % T::WI, pj = (e / T::WI) % T::WJ, vv = e / (T::WI * T::WJ);
@@ -1014,16 +1043,7 @@ __global__ void __launch_bounds__(InjSep<L>::NT)
       rj = ((rj % pn2) + pn2) % pn2;
       idx += (long long)rj * st2;
     }
-    float val = 0.0f;
-    if (ok) {
-      if (one_slot)  // the synchronous sub-step: t+1 only
-        val = w2 * h[((long long)s_p1 * nv + vv) * K + idx];
-      else
-        val = w0 * h[((long long)s_m1 * nv + vv) * K + idx] +
-              w1 * h[((long long)s_0 * nv + vv) * K + idx] +
-              w2 * h[((long long)s_p1 * nv + vv) * K + idx];
-    }
-    sv[vv][pj][pi] = val;
+    sv[vv][pj][pi] = ok ? h[vv * K + idx] : 0.0f;
   }
   __syncthreads();
   // along t1 (eq. spaceInt weights -1/16, 9/16, 9/16, -1/16 at odd child

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kFusedThreads, FUSED_MINB) k_fused(const __gri
           for (long long t = t0; t < n; t += stride) {
             const int run = (int)(t / R.K);
             capture_item<L, S>(T.v[l], R, ph.par, 0, ph.slot[0], ph.slot[0], T.ref,
-                               t - (long long)run * R.K, run);
+                               t - (long long)run * R.K, run, TimeInt{});
           }
           break;
         }

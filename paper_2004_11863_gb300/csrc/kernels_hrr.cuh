@@ -141,18 +141,8 @@ __global__ void k_parent_strain(LevelView p, LevelView c, RingDesc R, TnDesc T, 
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int run = blockIdx.y;
   if (k >= R.K) return;
-  const int fc = ring_face(R.start, R.nf, k);
-  long long loc = k - R.start[fc];
   int P[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int e = R.ext[fc][a];
-    const int i = (int)(loc % e);
-    loc /= e;
-    int cc = R.base[fc][a] + i;
-    if (R.pper[a]) cc = ((cc % R.pn[a]) + R.pn[a]) % R.pn[a];
-    P[a] = cc;
-  }
+  ring_node(R, k, P);
   const S* fp = run_cptr<S>(p, run);
   const S* fcb = run_cptr<S>(c, run);
   float up[3][3] = {}, um[3][3] = {};
@@ -199,13 +189,13 @@ __global__ void k_collide_bnd(LevelView c, BndDesc B, RingDesc R, const float* s
   const int run = blockIdx.y;
   if (k >= B.count) return;
   const int f = ring_face(B.start, B.nf, k);
-  long long loc = k - B.start[f];
+  unsigned loc = (unsigned)(k - B.start[f]);
   int X[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int e = B.ext[f][a];
-    X[a] = B.lo[f][a] + (int)(loc % e);
-    loc /= e;
+    const unsigned e = (unsigned)B.ext[f][a], q = loc / e;
+    X[a] = B.lo[f][a] + (int)(loc - q * e);
+    loc = q;
   }
   const int fa = B.axis[f];
   long long stride[3];

@@ -158,6 +158,14 @@ struct lbm_ctx {
   static constexpr int kPhases = 6;
   cudaGraphExec_t exec[kPhases] = {};
   long long exec_nodes[kPhases] = {};
+  // All phases as one graph, from phase 0: a graph launch costs about two
+  // microseconds on the device besides its kernels (five-kernel graphs of a
+  // small run: 1.64 us a kernel; thirty kernels in one graph: 1.22 us).
+  // Built the second time a call could use it, so that short runs do not
+  // pay for it.
+  cudaGraphExec_t exec_period = nullptr;
+  long long exec_period_nodes = 0;
+  bool period_seen = false;
   long long launches = 0;
   // per-kernel CUDA-event timing (lbm_profile)
   struct Rec {
@@ -279,6 +287,10 @@ Ops ops_for(int lattice) {
 
 void drop_graphs(lbm_ctx* h) {
   h->fused_valid = false;
+  if (h->exec_period) cudaGraphExecDestroy(h->exec_period);
+  h->exec_period = nullptr;
+  h->exec_period_nodes = 0;
+  h->period_seen = false;
   for (int k = 0; k < lbm_ctx::kPhases; ++k)
     if (h->exec[k]) {
       cudaGraphExecDestroy(h->exec[k]);
@@ -598,6 +610,129 @@ int sensor_pass(lbm_ctx* h, int l, int par, bool launch, bool with_velocity) {
   return LBM_OK;
 }
 
+// The capture's time interpolation for a child whose newest slot is c.head
+// (already rotated), and the slot a rebuild with weights wt then reads: the
+// interpolated one on the first sub-step, the newest on the second.
+TimeInt time_int(const Level& c, bool first) {
+  const float* w = first ? kTimeLin : kTimeQuad;
+  return TimeInt{1, (c.head + 1) % 3, (c.head + 2) % 3, w[0], w[1], w[2]};
+}
+int read_slot(const Level& v, const float* wt) {
+  return wt == kTimeDirect ? v.head : (v.head + 1) % 3;
+}
+
+// Lanes of special nodes when each takes several (an upper bound).
+constexpr long long EDGE_WIDE_MAX = 1LL << 20;
+
+// Whether level updates of this run take their special nodes along
+// (kernels_edge.cuh): 2D, not the hybrid collision, within the launch limits
+// on every level.
+bool edges_usable(const lbm_ctx* h) {
+  if (h->D != 2 || h->cfg.collision == LBM_HRR) return false;
+  for (int l = 0; l < h->nlev; ++l) {
+    const Level& v = h->lev[l];
+    long long items = l >= 1 ? v.bnd.count : 0;
+    if (l + 1 < h->nlev) items += h->lev[l + 1].tn.count;
+    const long long lanes = items * h->batch + EDGE_WIDE_MAX;
+    // (a slice of the update's grid holds at least 16 lanes per row)
+    if (lanes >= (1LL << 30) || lanes / (16LL * v.n[1]) + 1 + h->batch > 65535) return false;
+  }
+  return true;
+}
+
+bool any_sensors(const lbm_ctx* h) {
+  for (int l = 0; l < h->nlev; ++l)
+    if (h->lev[l].sens_on) return true;
+  return false;
+}
+
+// Description of level l's special nodes for its next update.
+Edge2d edge_desc(const lbm_ctx* h, int l, const float* wt) {
+  const Level& v = h->lev[l];
+  Edge2d E{};
+  if (l >= 1) {
+    const BndDesc& B = v.bnd;
+    const RingDesc& R = v.ring;
+    E.nb = (int)B.count;
+    E.nf = B.nf;
+    for (int f = 0; f < B.nf; ++f) {
+      E.b_axis[f] = B.axis[f];
+      E.b_side[f] = B.side[f];
+      E.b_start[f] = (int)B.start[f];
+      E.b_lo[f] = B.lo[f][1 - B.axis[f]];
+      E.r_start[f] = (int)R.start[f];
+    }
+    E.b_start[B.nf] = (int)B.count;
+    for (int a = 0; a < 2; ++a) {
+      E.p_boxed[a] = R.boxed[a];
+      E.p_n[a] = R.pn[a];
+    }
+    E.K = R.K;
+    E.run_stride = 3LL * R.nv * R.K;
+    E.hist = R.hist + (long long)read_slot(v, wt) * R.nv * R.K;
+    E.resc = (float)(v.tau / (2.0 * h->lev[l - 1].tau));  // eq. rescff
+  }
+  if (l + 1 < h->nlev) {
+    const Level& c = h->lev[l + 1];
+    const TnDesc& T = c.tn;
+    E.nt = (int)T.count;
+    E.tf = T.nf;
+    for (int f = 0; f < T.nf; ++f) {
+      E.t_axis[f] = T.axis[f];
+      E.t_start[f] = (int)T.start[f];
+      E.t_ra[f] = T.rlo[f][T.axis[f]];
+      E.t_lo[f] = T.rlo[f][1 - T.axis[f]];
+    }
+    E.t_start[T.nf] = (int)T.count;
+    for (int a = 0; a < 2; ++a) {
+      E.t_org[a] = T.lo[a];
+      E.t_boxed[a] = T.boxed[a];
+    }
+    E.child = c.view;
+    E.cpar = 1 - c.last;
+    E.t_resc = (float)(2.0 * v.tau / c.tau);  // eq. rescfc
+  }
+  return E;
+}
+
+// The level update of advance(): with sensors on, the special nodes were
+// rebuilt into the planes for the sensors to read; a 2D update takes them
+// along all the same, so that sensors change no bit of a run.
+cudaError_t update_op(lbm_ctx* h, int l, int par, const float* wt) {
+  const Level& v = h->lev[l];
+  if (edges_usable(h))
+    return h->ops.stream_collide_edges(v.view, h->cfg.collision, h->cfg.storage, par,
+                                       omega_of(v.tau), h->ref, v.k1_bx, v.k1_by,
+                                       edge_desc(h, l, wt), h->cur);
+  return h->ops.stream_collide(v.view, h->cfg.collision, h->cfg.storage, par, omega_of(v.tau),
+                               h->ref, v.k1_bx, v.k1_by, xf_of(h, l), h->cur);
+}
+
+// One step of level l of a 2D run whose updates take their special nodes
+// along: capture, child's first sub-step, this level's update (its TN nodes
+// read the child's state between its sub-steps), child's second sub-step --
+// one chain on one stream.
+int advance_edges(lbm_ctx* h, int l, const float* wt, bool launch) {
+  Level& v = h->lev[l];
+  const int st = h->cfg.storage;
+  const int par = 1 - v.last;
+  const bool child = l + 1 < h->nlev;
+  if (child) {
+    Level& c = h->lev[l + 1];
+    c.head = (c.head + 1) % 3;
+    LAUNCH_K(1, l, h->ops.capture(v.view, c.ring, st, par, 0, c.head, c.head,
+                                  time_int(c, v.nsteps == 0), h->ref, h->cur));
+    int rc = advance_edges(h, l + 1, v.nsteps == 0 ? kTimeLin : kTimeQuad, launch);
+    if (rc) return rc;
+  }
+  LAUNCH_K(0, l, h->ops.stream_collide_edges(v.view, h->cfg.collision, st, par, omega_of(v.tau),
+                                             h->ref, v.k1_bx, v.k1_by, edge_desc(h, l, wt),
+                                             h->cur));
+  v.last = par;
+  v.nsteps++;
+  return child ? advance_edges(h, l + 1, kTimeDirect, launch) : LBM_OK;
+}
+
 // One step of level l with its finer levels (see the file comment).
 int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_before_update) {
   Level& v = h->lev[l];
@@ -611,7 +746,7 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
     if (h->recording)
       h->recording->push_back(Phase{2, l, par, 0, {slots[0], slots[1], slots[2]},
                                     {wt[0], wt[1], wt[2]}, resc, 0.0f});
-    LAUNCH_K(2, l, h->ops.inject(v.view, v.bnd, v.ring, st, wt, slots, resc, par, ref,
+    LAUNCH_K(2, l, h->ops.inject(v.view, v.bnd, v.ring, st, read_slot(v, wt), resc, par, ref,
                                  xf_of(h, l), h->cur));
   }
   if (l + 1 < h->nlev) {
@@ -619,7 +754,8 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
     c.head = (c.head + 1) % 3;
     if (h->recording)
       h->recording->push_back(Phase{1, l, par, 0, {c.head, c.head, c.head}, {}, 0.0f, 0.0f});
-    LAUNCH_K(1, l, h->ops.capture(v.view, c.ring, st, par, 0, c.head, c.head, ref, h->cur));
+    LAUNCH_K(1, l, h->ops.capture(v.view, c.ring, st, par, 0, c.head, c.head,
+                                  time_int(c, v.nsteps == 0), ref, h->cur));
     int rc = advance(h, l + 1, v.nsteps == 0 ? kTimeLin : kTimeQuad, launch, nullptr);
     if (rc) return rc;
     // The restriction and level l's own update need nothing the child's
@@ -653,8 +789,9 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
     // no barrier before the child's next phase: nothing there reads or
     // writes this level's populations)
     const Phase upd{0, l, par, 0, {}, {}, 0.0f, omega_of(v.tau), 1};
-    LAUNCH_K(0, l, h->ops.stream_collide(v.view, h->cfg.collision, st, par, omega_of(v.tau), ref,
-                                         v.k1_bx, v.k1_by, xf_of(h, l), h->cur));
+    LAUNCH_K(0, l, update_op(h, l, par, wt));
+    // (a 2D update reads the child's state between its sub-steps itself)
+    if (fork && edges_usable(h)) CK(cudaEventRecord(h->ev_restrict[l], h->side[l]));
     if (fork) {
       CK(cudaEventRecord(h->ev_join[l], h->side[l]));
       h->cur = main;
@@ -672,8 +809,7 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
   if (rs) return rs;
   if (launch && wait_before_update) CK(cudaStreamWaitEvent(h->cur, wait_before_update, 0));
   if (h->recording) h->recording->push_back(Phase{0, l, par, 0, {}, {}, 0.0f, omega_of(v.tau)});
-  LAUNCH_K(0, l, h->ops.stream_collide(v.view, h->cfg.collision, st, par, omega_of(v.tau), ref,
-                                       v.k1_bx, v.k1_by, xf_of(h, l), h->cur));
+  LAUNCH_K(0, l, update_op(h, l, par, wt));
   v.last = par;
   v.nsteps++;
   return LBM_OK;
@@ -706,13 +842,14 @@ int advance_hrr(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wai
     slots[0] = (v.head + 1) % 3;
     slots[1] = (v.head + 2) % 3;
     slots[2] = v.head;
-    LAUNCH_K(2, l, h->ops.inject(v.view, v.bnd, v.ring, st, wt, slots, resc, par, ref, nullptr,
-                                 h->cur));
+    LAUNCH_K(2, l, h->ops.inject(v.view, v.bnd, v.ring, st, read_slot(v, wt), resc, par, ref,
+                                 nullptr, h->cur));
   }
   if (l + 1 < h->nlev) {
     Level& c = h->lev[l + 1];
     c.head = (c.head + 1) % 3;
-    LAUNCH_K(1, l, h->ops.capture(v.view, c.ring, st, par, 0, c.head, c.head, ref, h->cur));
+    LAUNCH_K(1, l, h->ops.capture(v.view, c.ring, st, par, 0, c.head, c.head,
+                                  time_int(c, v.nsteps == 0), ref, h->cur));
     int rc = advance_hrr(h, l + 1, v.nsteps == 0 ? kTimeLin : kTimeQuad, launch, nullptr, true);
     if (rc) return rc;
     cudaStream_t main = h->cur;
@@ -777,8 +914,11 @@ int probe_launch(lbm_ctx* h, bool launch) {
 }
 
 int coarse_step(lbm_ctx* h, bool launch) {
-  int rc = h->cfg.collision == LBM_HRR ? advance_hrr(h, 0, nullptr, launch, nullptr, false)
-                                       : advance(h, 0, nullptr, launch, nullptr);
+  // (the fused step's programs are recorded from the per-operation schedule)
+  int rc = h->cfg.collision == LBM_HRR        ? advance_hrr(h, 0, nullptr, launch, nullptr, false)
+           : !h->recording && !any_sensors(h) && edges_usable(h)
+               ? advance_edges(h, 0, nullptr, launch)
+                                              : advance(h, 0, nullptr, launch, nullptr);
   if (rc) return rc;
   return probe_launch(h, launch);
 }
@@ -791,8 +931,8 @@ int seed_history(lbm_ctx* h) {
   for (int l = 1; l < h->nlev; ++l) {
     Level& p = h->lev[l - 1];
     h->lev[l].head = 1;
-    LAUNCH(h->ops.capture(p.view, h->lev[l].ring, h->cfg.storage, p.last, 1, 1, 0, h->ref,
-                          h->cur));
+    LAUNCH(h->ops.capture(p.view, h->lev[l].ring, h->cfg.storage, p.last, 1, 1, 0, TimeInt{},
+                          h->ref, h->cur));
     if (h->cfg.collision == LBM_HRR)
       LAUNCH(h->ops.parent_strain(p.view, h->lev[l].view, h->lev[l].ring, h->lev[l].tn,
                                   h->cfg.storage, (float*)h->lev[l].sh_mem, 1, 0, p.last,
@@ -1348,6 +1488,45 @@ int lbm_set_fused(lbm_handle h, int mode) {
   return LBM_OK;
 }
 
+namespace {
+
+// n coarse steps by replaying *exec, captured first if it does not exist yet
+// (the capture advances the host bookkeeping like the steps themselves).
+int replay(lbm_ctx* h, int n, cudaGraphExec_t* exec, long long* nodes) {
+  if (!*exec) {
+    cudaGraph_t g = nullptr;
+    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+    h->cur = h->cap_stream;
+    const long long before = h->launches;
+    int rc = LBM_OK;
+    for (int k = 0; k < n && rc == LBM_OK; ++k) rc = coarse_step(h, true);
+    cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
+    h->cur = h->stream;
+    h->launches = before;  // counted when the graph runs
+    if (rc) {
+      if (g) cudaGraphDestroy(g);
+      return rc;
+    }
+    CK(e);
+    size_t nn = 0;
+    cudaGraphGetNodes(g, nullptr, &nn);
+    e = cudaGraphInstantiate(exec, g, 0);
+    cudaGraphDestroy(g);
+    CK(e);
+    *nodes = (long long)nn;
+  } else {
+    for (int k = 0; k < n; ++k) {
+      int rc = coarse_step(h, false);
+      if (rc) return rc;
+    }
+  }
+  CK(cudaGraphLaunch(*exec, h->stream));
+  h->launches += *nodes;
+  return LBM_OK;
+}
+
+}  // namespace
+
 int lbm_step(lbm_handle h, int n_coarse) {
   if (!h || n_coarse < 0) return LBM_EINVAL;
   if (!h->ready) return LBM_ESTATE;
@@ -1355,47 +1534,31 @@ int lbm_step(lbm_handle h, int n_coarse) {
     int rc = seed_history(h);
     if (rc) return rc;
   }
-  for (int s = 0; s < n_coarse; ++s) {
+  int done = 1;  // coarse steps taken by one pass of the loop
+  for (int s = 0; s < n_coarse; s += done) {
+    done = 1;
     // the first coarse step (first sub-steps with one history slot) stays
     // on the per-phase kernels; the fused programs start after it
     if (h->coarse_steps > 0 && fused_usable(h)) return fused_steps(h, n_coarse - s);
+    int rc = LBM_OK;
     if (h->coarse_steps == 0 || !h->use_graphs || h->profiling) {
       h->cur = h->stream;
-      int rc = coarse_step(h, true);
-      if (rc) return rc;
+      rc = coarse_step(h, true);
     } else {
       // every level's parity and every history rotation restart with the
       // initial state, so the phase of a coarse step is its index mod 6
       const int key = (int)(h->coarse_steps % lbm_ctx::kPhases);
-      if (!h->exec[key]) {
-        cudaGraph_t g = nullptr;
-        CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-        h->cur = h->cap_stream;
-        const long long before = h->launches;
-        int rc = coarse_step(h, true);
-        cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
-        h->cur = h->stream;
-        h->launches = before;  // counted when the graph runs
-        if (rc) {
-          if (g) cudaGraphDestroy(g);
-          return rc;
-        }
-        CK(e);
-        size_t nn = 0;
-        cudaGraphGetNodes(g, nullptr, &nn);
-        e = cudaGraphInstantiate(&h->exec[key], g, 0);
-        cudaGraphDestroy(g);
-        CK(e);
-        h->exec_nodes[key] = (long long)nn;
+      if (key == 0 && n_coarse - s >= lbm_ctx::kPhases && h->period_seen) {
+        done = lbm_ctx::kPhases;
+        rc = replay(h, done, &h->exec_period, &h->exec_period_nodes);
       } else {
-        int rc = coarse_step(h, false);
-        if (rc) return rc;
+        h->period_seen = h->period_seen || (key == 0 && n_coarse - s >= lbm_ctx::kPhases);
+        rc = replay(h, 1, &h->exec[key], &h->exec_nodes[key]);
       }
-      CK(cudaGraphLaunch(h->exec[key], h->stream));
-      h->launches += h->exec_nodes[key];
     }
-    ++h->coarse_steps;
-    if (h->probe_n > 0) ++h->probe_pending;
+    if (rc) return rc;
+    h->coarse_steps += done;
+    if (h->probe_n > 0) h->probe_pending += done;
   }
   return LBM_OK;
 }

@@ -26,96 +26,121 @@ RefF make_ref_f(const RefState& r) {
   return R;
 }
 
+// Prepends the z-slices of special blocks to a 2D update's grid
+// (kernels_edge.cuh).  First in the grid, so that their longer chain of loads
+// runs beside the plain blocks and not after them.  Several lanes a node up
+// to EDGE_WIDE_LANES of them, about what the GPU holds beside the plain
+// blocks (kernels_edge.cuh has both sides measured).
+template <class L>
+NoEdge<L> with_slices(const NoEdge<L>& E, int, dim3&, const dim3&) {
+  return E;
+}
+#ifndef EDGE_WIDE_LANES
+#define EDGE_WIDE_LANES 65536
+#endif
+inline Edge2d with_slices(Edge2d E, int batch, dim3& grid, const dim3& block) {
+  E.wide = (4LL * E.nb + 16LL * E.nt) * batch <= EDGE_WIDE_LANES;
+  const long long bl = ((long long)E.nb * batch * (E.wide ? 4 : 1) + 31) / 32 * 32;
+  const long long lanes = bl + (long long)E.nt * batch * (E.wide ? 16 : 1);
+  const long long slice = (long long)grid.x * grid.y * block.x * block.y;
+  E.nz = (int)((lanes + slice - 1) / slice);
+  grid.z += E.nz;
+  return E;
+}
+
 template <class L, class S, int COLL>
 cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx,
-                         int by, const S* xf, cudaStream_t s) {
+                         int by, const S* xf, const EdgeArg<L>& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   if (v.run_stride >= (1LL << 31)) return cudaErrorInvalidValue;  // (32-bit offsets)
   dim3 block(bx, by, 1);
   dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + 2 * by - 1) / (2 * by),
             (v.n[2] + K1X2Pfz<S>::PZ - 1) / K1X2Pfz<S>::PZ * v.batch);
+  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   if (mov) {
     if (par == 0)
-      k_stream_collide_x2<L, S, COLL, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_x2<L, S, COLL, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide_x2<L, S, COLL, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_x2<L, S, COLL, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   } else {
     if (par == 0)
-      k_stream_collide_x2<L, S, COLL, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_x2<L, S, COLL, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide_x2<L, S, COLL, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_x2<L, S, COLL, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   }
   return cudaGetLastError();
 }
 
 template <class L, class S, int COLL>
 cudaError_t sc_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx, int by,
-                      const S* xf, cudaStream_t s) {
+                      const S* xf, const EdgeArg<L>& E, cudaStream_t s) {
   // (the two-node update addresses a run with 32-bit offsets: larger runs
   // take the one-node update)
   if constexpr ((std::is_same<S, float>::value && K1X2Tune<L>::ON) ||
                 (std::is_same<S, __half>::value && K1X2Tune<L>::ON_H))
-    if (v.run_stride < (1LL << 31)) return sc_x2_launch<L, S, COLL>(v, par, omega, ref, bx, by, xf, s);
+    if (v.run_stride < (1LL << 31)) return sc_x2_launch<L, S, COLL>(v, par, omega, ref, bx, by, xf, E, s);
   constexpr int NPT = K1Tune<L, S>::NPT;
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   dim3 block(bx, by, 1);
   dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + by * NPT - 1) / (by * NPT), v.n[2] * v.batch);
+  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   if (mov) {
     if (par == 0)
-      k_stream_collide<L, COLL, S, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide<L, COLL, S, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide<L, COLL, S, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide<L, COLL, S, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   } else {
     if (par == 0)
-      k_stream_collide<L, COLL, S, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide<L, COLL, S, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide<L, COLL, S, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide<L, COLL, S, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   }
   return cudaGetLastError();
 }
 
 template <class L, int COLL>
 cudaError_t sc_pair_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx,
-                           int by, const __half* xf, cudaStream_t s) {
+                           int by, const __half* xf, const EdgeArg<L>& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   dim3 block(bx, by, 1);
   dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + by - 1) / by, v.n[2] * ((v.batch + 1) / 2));
+  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   if (mov) {
     if (par == 0)
-      k_stream_collide_pair<L, COLL, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_pair<L, COLL, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide_pair<L, COLL, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_pair<L, COLL, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   } else {
     if (par == 0)
-      k_stream_collide_pair<L, COLL, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_pair<L, COLL, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide_pair<L, COLL, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf);
+      k_stream_collide_pair<L, COLL, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
   }
   return cudaGetLastError();
 }
 
 template <class L, class S>
 cudaError_t sc_coll(const LevelView& v, int coll, int par, float omega, const RefState& ref,
-                    int bx, int by, const void* xf, cudaStream_t s) {
+                    int bx, int by, const void* xf, const EdgeArg<L>& E, cudaStream_t s) {
   const S* xs = static_cast<const S*>(xf);
   if (std::is_same<S, __half>::value && v.es == 2) {
     const __half* xh = static_cast<const __half*>(xf);
     switch (coll) {
-      case 0: return sc_pair_launch<L, 0>(v, par, omega, ref, bx, by, xh, s);
-      case 1: return sc_pair_launch<L, 1>(v, par, omega, ref, bx, by, xh, s);
-      default: return sc_pair_launch<L, 2>(v, par, omega, ref, bx, by, xh, s);
+      case 0: return sc_pair_launch<L, 0>(v, par, omega, ref, bx, by, xh, E, s);
+      case 1: return sc_pair_launch<L, 1>(v, par, omega, ref, bx, by, xh, E, s);
+      default: return sc_pair_launch<L, 2>(v, par, omega, ref, bx, by, xh, E, s);
     }
   }
   switch (coll) {
-    case 0: return sc_launch<L, S, 0>(v, par, omega, ref, bx, by, xs, s);
-    case 1: return sc_launch<L, S, 1>(v, par, omega, ref, bx, by, xs, s);
-    default: return sc_launch<L, S, 2>(v, par, omega, ref, bx, by, xs, s);
+    case 0: return sc_launch<L, S, 0>(v, par, omega, ref, bx, by, xs, E, s);
+    case 1: return sc_launch<L, S, 1>(v, par, omega, ref, bx, by, xs, E, s);
+    default: return sc_launch<L, S, 2>(v, par, omega, ref, bx, by, xs, E, s);
   }
 }
 
@@ -123,26 +148,38 @@ template <class L>
 cudaError_t stream_collide(const LevelView& v, int coll, int storage, int par, float omega,
                            const RefState& ref, int bx, int by, const void* xf,
                            cudaStream_t s) {
-  return storage == 0 ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, xf, s)
-                      : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, xf, s);
+  return storage == 0 ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, xf, EdgeArg<L>{}, s)
+                      : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, xf, EdgeArg<L>{}, s);
+}
+
+// The 2D update with its special nodes (E.nb, E.nt of them per run).
+template <class L>
+cudaError_t stream_collide_edges(const LevelView& v, int coll, int storage, int par, float omega,
+                                 const RefState& ref, int bx, int by, const Edge2d& E,
+                                 cudaStream_t s) {
+  if constexpr (L::D == 2)
+    return storage == 0
+               ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, nullptr, E, s)
+               : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, nullptr, E, s);
+  return cudaErrorInvalidValue;
 }
 
 template <class L>
 cudaError_t capture(const LevelView& p, const RingDesc& R, int storage, int par, int mode,
-                    int s_new, int s_also, const RefState& ref, cudaStream_t s) {
+                    int s_new, int s_also, const TimeInt& ti, const RefState& ref,
+                    cudaStream_t s) {
   if (R.K == 0) return cudaSuccess;
   dim3 grid(blocks_for(R.K, 64), p.batch);
   if (storage == 0)
-    k_capture<L, float><<<grid, 64, 0, s>>>(p, R, par, mode, s_new, s_also, make_ref_f<L>(ref));
+    k_capture<L, float><<<grid, 64, 0, s>>>(p, R, par, mode, s_new, s_also, ti, make_ref_f<L>(ref));
   else
-    k_capture<L, __half><<<grid, 64, 0, s>>>(p, R, par, mode, s_new, s_also, make_ref_f<L>(ref));
+    k_capture<L, __half><<<grid, 64, 0, s>>>(p, R, par, mode, s_new, s_also, ti, make_ref_f<L>(ref));
   return cudaGetLastError();
 }
 
 template <class L>
 cudaError_t inject(const LevelView& c, const BndDesc& B, const RingDesc& R, int storage,
-                   const float* wt, const int* slots, float resc, int par, const RefState& ref,
-                   void* xf, cudaStream_t s) {
+                   int slot, float resc, int par, const RefState& ref, void* xf, cudaStream_t s) {
   if (B.count == 0) return cudaSuccess;
   using T = InjTile<L>;
   InjDesc J{};
@@ -168,23 +205,19 @@ cudaError_t inject(const LevelView& c, const BndDesc& B, const RingDesc& R, int 
   if constexpr (L::D == 3) {
     dim3 block(T::TI, T::TJ);
     if (storage == 0)
-      k_inject_sep<L, float><<<grid, block, 0, s>>>(c, J, R, wt[0], wt[1], wt[2], slots[0],
-                                                    slots[1], slots[2], resc, par,
-                                                    make_ref_f<L>(ref), static_cast<float*>(xf));
+      k_inject_sep<L, float><<<grid, block, 0, s>>>(c, J, R, slot, resc, par, make_ref_f<L>(ref),
+                                                    static_cast<float*>(xf));
     else
-      k_inject_sep<L, __half><<<grid, block, 0, s>>>(c, J, R, wt[0], wt[1], wt[2], slots[0],
-                                                     slots[1], slots[2], resc, par,
+      k_inject_sep<L, __half><<<grid, block, 0, s>>>(c, J, R, slot, resc, par,
                                                      make_ref_f<L>(ref), static_cast<__half*>(xf));
     return cudaGetLastError();
   }
   dim3 block(T::TI, T::TJ, T::G);
   if (storage == 0)
-    k_inject<L, float><<<grid, block, 0, s>>>(c, J, R, wt[0], wt[1], wt[2], slots[0], slots[1],
-                                              slots[2], resc, par, make_ref_f<L>(ref),
+    k_inject<L, float><<<grid, block, 0, s>>>(c, J, R, slot, resc, par, make_ref_f<L>(ref),
                                               static_cast<float*>(xf));
   else
-    k_inject<L, __half><<<grid, block, 0, s>>>(c, J, R, wt[0], wt[1], wt[2], slots[0], slots[1],
-                                               slots[2], resc, par, make_ref_f<L>(ref),
+    k_inject<L, __half><<<grid, block, 0, s>>>(c, J, R, slot, resc, par, make_ref_f<L>(ref),
                                                static_cast<__half*>(xf));
   return cudaGetLastError();
 }
@@ -472,6 +505,7 @@ Ops make_ops() {
   o.q = L::Q;
   o.d = L::D;
   o.stream_collide = detail::stream_collide<L>;
+  o.stream_collide_edges = detail::stream_collide_edges<L>;
   o.capture = detail::capture<L>;
   o.inject = detail::inject<L>;
   o.restrict_tn = detail::restrict_tn<L>;
