@@ -431,12 +431,13 @@ __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
 #ifndef K1X2_MINB_D3Q27
 #define K1X2_MINB_D3Q27 3
 #endif
-// MINB1: resident blocks of the binary32 odd-parity update, whose shifted
-// addresses need more registers: at the even update's bound it spilled
-// (D3Q19: 104 bytes at 128 registers); one block fewer holds it in
-// registers (D3Q19 168, D3Q27 252), +3 % on the D3Q19 slab's step and +2 %
-// on the nested D3Q27 case (GB300); both parities at the lower bound were
-// slower.
+// MINB1: resident blocks of the binary32 odd-parity update; its shifted
+// addresses need more registers, but without the warps' one-node row ends the
+// even update's bound holds them (GB300, D3Q19 slab 4.22 -> 4.12 ms a step
+// against one block fewer, nested D3Q27 2.40 -> 2.35 ms) -- except for the
+// BGK collision, which keeps the populations to the end and spills there
+// (K1X2_MINB1_BGK_<lattice>; a D3Q27 level of 161 x 97 x 83 nodes: 57 us a
+// step, 70 at the even update's bound).
 #ifndef K1X2H_MINB1_D2Q9
 #define K1X2H_MINB1_D2Q9 K1X2H_MINB_D2Q9
 #endif
@@ -450,10 +451,31 @@ __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
 #define K1X2_MINB1_D2Q9 K1X2_MINB_D2Q9
 #endif
 #ifndef K1X2_MINB1_D3Q19
-#define K1X2_MINB1_D3Q19 3
+#define K1X2_MINB1_D3Q19 4
 #endif
 #ifndef K1X2_MINB1_D3Q27
-#define K1X2_MINB1_D3Q27 2
+#define K1X2_MINB1_D3Q27 3
+#endif
+// (with a face buffer, whose instance needs fewer registers; 302 -> 268 us
+// on the finest level of the nested D3Q27 case at four blocks, levels without
+// one 222 -> 253)
+#ifndef K1X2_MINB1_XF_D3Q27
+#define K1X2_MINB1_XF_D3Q27 4
+#endif
+#ifndef K1X2_MINB1_XF_D3Q19
+#define K1X2_MINB1_XF_D3Q19 K1X2_MINB1_D3Q19
+#endif
+#ifndef K1X2_MINB1_XF_D2Q9
+#define K1X2_MINB1_XF_D2Q9 K1X2_MINB1_D2Q9
+#endif
+#ifndef K1X2_MINB1_BGK_D3Q19
+#define K1X2_MINB1_BGK_D3Q19 3
+#endif
+#ifndef K1X2_MINB1_BGK_D3Q27
+#define K1X2_MINB1_BGK_D3Q27 2
+#endif
+#ifndef K1X2_MINB1_BGK_D2Q9
+#define K1X2_MINB1_BGK_D2Q9 K1X2_MINB1_D2Q9
 #endif
 template <class L>
 struct K1X2Tune;
@@ -463,6 +485,8 @@ struct K1X2Tune<D2Q9> {
   static constexpr bool ON_H = K1X2H_D2Q9;
   static constexpr int MINB = K1X2_MINB_D2Q9;
   static constexpr int MINB1 = K1X2_MINB1_D2Q9;
+  static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D2Q9;
+  static constexpr int MINB1_XF = K1X2_MINB1_XF_D2Q9;
   static constexpr int MINB_H = K1X2H_MINB_D2Q9;
   static constexpr int MINB1_H = K1X2H_MINB1_D2Q9;
 };
@@ -472,6 +496,8 @@ struct K1X2Tune<D3Q19> {
   static constexpr bool ON_H = K1X2H_D3Q19;
   static constexpr int MINB = K1X2_MINB_D3Q19;
   static constexpr int MINB1 = K1X2_MINB1_D3Q19;
+  static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D3Q19;
+  static constexpr int MINB1_XF = K1X2_MINB1_XF_D3Q19;
   static constexpr int MINB_H = K1X2H_MINB_D3Q19;
   static constexpr int MINB1_H = K1X2H_MINB1_D3Q19;
 };
@@ -481,6 +507,8 @@ struct K1X2Tune<D3Q27> {
   static constexpr bool ON_H = K1X2H_D3Q27;
   static constexpr int MINB = K1X2_MINB_D3Q27;
   static constexpr int MINB1 = K1X2_MINB1_D3Q27;
+  static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D3Q27;
+  static constexpr int MINB1_XF = K1X2_MINB1_XF_D3Q27;
   static constexpr int MINB_H = K1X2H_MINB_D3Q27;
   static constexpr int MINB1_H = K1X2H_MINB1_D3Q27;
 };
@@ -489,20 +517,48 @@ struct K1X2Tune<D3Q27> {
 // more: the thread walks that many consecutive planes and prefetches the
 // next plane's populations into L2 before colliding the current one, which
 // keeps DRAM reads in flight during the collision without holding
-// registers).  Binary32: 8 planes (against one: +9 % on the D3Q19 slab;
-// against four: +1.3 % there and +1 % on the nested D3Q27 case; sixteen
-// measured no better); binary16: 1 (its update is nearer the instruction
-// limit: the prefetches cost it 5-7 %).  Measured on GB300.
-#ifndef K1X2_PFZ_F
-#define K1X2_PFZ_F 8
+// registers).  Binary32: D3Q19 8 planes (against one: +9 % on the slab;
+// against four: +0.8 %; sixteen, -2 %), D3Q27 4 (against eight: +1 % on the
+// nested case, +7 % on a 161 x 97 x 83 level; two, -1 %); binary16: 1 (its
+// update is nearer the instruction limit: with four planes the slab's step
+// takes 937 us, not 860).  Measured on GB300.
+#ifndef K1X2_PFZ_19F
+#define K1X2_PFZ_19F 8
+#endif
+#ifndef K1X2_PFZ_27F
+#define K1X2_PFZ_27F 4
 #endif
 #ifndef K1X2_PFZ_H
 #define K1X2_PFZ_H 1
 #endif
-template <class S>
+template <class L, class S>
 struct K1X2Pfz {
-  static constexpr int PZ = std::is_same<S, float>::value ? K1X2_PFZ_F : K1X2_PFZ_H;
+  static constexpr int PZ = !std::is_same<S, float>::value ? K1X2_PFZ_H
+                            : L::Q == 27                   ? K1X2_PFZ_27F
+                                                           : K1X2_PFZ_19F;
 };
+
+// Node (x, y) at element e of a 3D level's z-plane, counted from its first
+// node (the two-node update: of its even rows; the odd ones are the other
+// lane's).  The 3D updates walk a plane's elements, not its rows: a refined
+// level has 2 E + 1 nodes in a row, so rows cut into warps leave a warp of
+// one lane at the end of each (a ninth one for 257 nodes), and rows padded to
+// whole cache lines leave a line of one node.  3D rows are padded to whole
+// sectors only (build_view), and warps run across their ends; elements
+// between rows (ghost nodes, padding) are idle lanes (x >= n[0]).  One
+// periodic level of 257 x 512 x 256 nodes (D3Q19) 868 -> 829 us, 193 x 192^2
+// (D3Q27) 285 -> 273, 161 x 160^2 in binary16 82 -> 76; 256- and 192-node
+// rows as before.
+__device__ __forceinline__ void plane_node(const LevelView& v, unsigned e, int& x, int& y) {
+  const unsigned r = e / (unsigned)v.SX;
+  y = (int)r;
+  x = (int)(e - r * (unsigned)v.SX);
+}
+
+// Whether a lane of the warp lies on a face normal to x.
+__device__ __forceinline__ bool warp_has_xface(const LevelView& v, int x) {
+  return __any_sync(__activemask(), x == 0 || x == v.n[0] - 1);
+}
 
 // Element offsets of the two-node update within a run are 32-bit (the
 // launcher takes it only for runs below 2^31 elements; larger runs take the
@@ -513,7 +569,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-template <class L, class S, int COLL, int PAR, bool MOV>
+// XF: the level has a face buffer, xf.
+template <class L, class S, int COLL, int PAR, bool MOV, bool XF>
 __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float omega,
                                                        const RefF& R, const S* __restrict__ xf,
                                                        const EdgeArg<L>& E, int x, int y0, int z,
@@ -525,38 +582,42 @@ __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float
   // each lane's node; an idle lane reads its partner's
   const NodeAddr a0 = node_addr<L>(v, x, ok0 ? y0 : y0 + 1, z);
   const NodeAddr a1 = node_addr<L>(v, x, ok1 ? y0 + 1 : y0, z);
-  // a lane on a face normal to x takes its populations from the face buffer:
-  // every lane loads from the planes, then only warps holding such a lane
-  // (a warp-uniform branch) replace that lane's values by the face buffer's
-  const bool fw = warp_has_xface(v, xf);
-  const bool fx = fw && (x == 0 || x == v.n[0] - 1);
   // element offsets are formed whole before indexing (f[i * plane + at]):
   // per-direction base pointers would cost 64-bit registers per direction
   F2 g[L::Q];
-  sfor<L::Q>([&](auto I) {
+  auto plane_at = [&](auto I, const NodeAddr& a) {
     constexpr int i = decltype(I)::value;
-    if constexpr (PAR == 0) {
-      g[i].v.x = Store<S>::ld(&f[(X2Idx)i * (X2Idx)v.plane + a0.at(0, 0, 0)]);
-      g[i].v.y = Store<S>::ld(&f[(X2Idx)i * (X2Idx)v.plane + a1.at(0, 0, 0)]);
-    } else {
-      g[i].v.x = Store<S>::ld(
-          &f[(X2Idx)opp<L>(i) * (X2Idx)v.plane + a0.at(-L::c(i, 0), -L::c(i, 1), -L::c(i, 2))]);
-      g[i].v.y = Store<S>::ld(
-          &f[(X2Idx)opp<L>(i) * (X2Idx)v.plane + a1.at(-L::c(i, 0), -L::c(i, 1), -L::c(i, 2))]);
-    }
-  });
-  if constexpr (L::D == 3) {  // (2D levels have no face buffer)
-    if (fw && fx) {
-      const long long F = (long long)v.n[1] * v.n[2];
-      const S* xb = xf + ((long long)run * 2 + (x != 0)) * L::Q * F + (long long)z * v.n[1];
-      const S* xb0 = xb + (ok0 ? y0 : y0 + 1);
-      const S* xb1 = xb + (ok1 ? y0 + 1 : y0);
-      sfor<L::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        g[i].v.x = Store<S>::ld(xb0 + i * F);
-        g[i].v.y = Store<S>::ld(xb1 + i * F);
-      });
-    }
+    if constexpr (PAR == 0)
+      return &f[(X2Idx)i * (X2Idx)v.plane + a.at(0, 0, 0)];
+    else
+      return &f[(X2Idx)opp<L>(i) * (X2Idx)v.plane + a.at(-L::c(i, 0), -L::c(i, 1), -L::c(i, 2))];
+  };
+  // A node on a face normal to x takes its populations from the face buffer.
+  // Warps that hold one choose each lane's address (a warp-uniform branch:
+  // the others run the plain loads); loading from the planes first and
+  // replacing those lanes' values made a face warp wait for DRAM twice, as
+  // the second load of a register waits for the first (finest level of the
+  // nested D3Q27 case 311 -> 298 us, D3Q19 slab 1777 -> 1741).  Levels without
+  // a face buffer have an instance without the choice, which costs them 3 %.
+  bool face_warp = false;
+  if constexpr (XF) face_warp = warp_has_xface(v, x);
+  if (face_warp) {
+    const bool fx = x == 0 || x == v.n[0] - 1;
+    const long long F = (long long)v.n[1] * v.n[2];
+    const S* xb = xf + ((long long)run * 2 + (x != 0)) * L::Q * F + (long long)z * v.n[1];
+    const S* xb0 = xb + (ok0 ? y0 : y0 + 1);
+    const S* xb1 = xb + (ok1 ? y0 + 1 : y0);
+    sfor<L::Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      g[i].v.x = Store<S>::ld(fx ? xb0 + i * F : plane_at(I, a0));
+      g[i].v.y = Store<S>::ld(fx ? xb1 + i * F : plane_at(I, a1));
+    });
+  } else {
+    sfor<L::Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      g[i].v.x = Store<S>::ld(plane_at(I, a0));
+      g[i].v.y = Store<S>::ld(plane_at(I, a1));
+    });
   }
   collide_emit<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
     constexpr int i = decltype(I)::value;
@@ -574,28 +635,37 @@ __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float
   });
 }
 
-template <class L, class S, int COLL, int PAR, bool MOV>
-__global__ void __launch_bounds__(128, std::is_same<S, float>::value
-                                           ? (PAR ? K1X2Tune<L>::MINB1 : K1X2Tune<L>::MINB)
-                                           : (PAR ? K1X2Tune<L>::MINB1_H : K1X2Tune<L>::MINB_H))
+template <class L, class S, int COLL, int PAR, bool MOV, bool XF>
+__global__ void __launch_bounds__(128, !std::is_same<S, float>::value
+                                           ? (PAR ? K1X2Tune<L>::MINB1_H : K1X2Tune<L>::MINB_H)
+                                       : PAR == 0  ? K1X2Tune<L>::MINB
+                                       : COLL == 0 ? K1X2Tune<L>::MINB1_BGK
+                                       : XF        ? K1X2Tune<L>::MINB1_XF
+                                                   : K1X2Tune<L>::MINB1)
     k_stream_collide_x2(LevelView v, float omega, RefF R, const S* __restrict__ xf,
                         const __grid_constant__ EdgeArg<L> E) {
-  constexpr int PZ = K1X2Pfz<S>::PZ;
+  constexpr int PZ = K1X2Pfz<L, S>::PZ;
   if (edge_block<L, S, COLL, PAR, MOV>(v, omega, R, E)) return;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * 2;
   const int nzb = (v.n[2] + PZ - 1) / PZ;  // z blocks per run
   int zc = blockIdx.z - edge_slices(E), run = 0;
   if (v.batch > 1) {
     run = zc / nzb;
     zc -= run * nzb;
   }
-  if (x >= v.n[0]) return;
+  int x, y0;
+  if constexpr (L::D == 3) {
+    plane_node(v, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y0);
+    y0 *= 2;
+  } else {
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y0 = (blockIdx.y * blockDim.y + threadIdx.y) * 2;
+  }
+  if (x >= v.n[0] || y0 >= v.n[1]) return;
   if constexpr (PZ == 1) {
-    stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, E, x, y0, zc, run);
+    stream_collide_x2_pair<L, S, COLL, PAR, MOV, XF>(v, omega, R, xf, E, x, y0, zc, run);
   } else {
     const S* f = static_cast<const S*>(v.f) + run * v.run_stride;
-    const int ya = y0 < v.n[1] ? y0 : v.n[1] - 1, yb = y0 + 1 < v.n[1] ? y0 + 1 : ya;
+    const int yb = y0 + 1 < v.n[1] ? y0 + 1 : y0;
 #pragma unroll 1
     for (int k = 0; k < PZ; ++k) {
       const int z = zc * PZ + k;
@@ -603,8 +673,8 @@ __global__ void __launch_bounds__(128, std::is_same<S, float>::value
       // the next plane's populations into L2 (not for nodes a parent level
       // leaves to its child: they are not updated)
       if (k + 1 < PZ && z + 1 < v.n[2] &&
-          !(inactive(v, x, ya, z + 1) && inactive(v, x, yb, z + 1))) {
-        const NodeAddr p0 = node_addr<L>(v, x, ya, z + 1), p1 = node_addr<L>(v, x, yb, z + 1);
+          !(inactive(v, x, y0, z + 1) && inactive(v, x, yb, z + 1))) {
+        const NodeAddr p0 = node_addr<L>(v, x, y0, z + 1), p1 = node_addr<L>(v, x, yb, z + 1);
         sfor<L::Q>([&](auto I) {
           constexpr int i = decltype(I)::value;
           if constexpr (PAR == 0) {
@@ -618,7 +688,7 @@ __global__ void __launch_bounds__(128, std::is_same<S, float>::value
           }
         });
       }
-      stream_collide_x2_pair<L, S, COLL, PAR, MOV>(v, omega, R, xf, E, x, y0, z, run);
+      stream_collide_x2_pair<L, S, COLL, PAR, MOV, XF>(v, omega, R, xf, E, x, y0, z, run);
     }
   }
 }
@@ -659,8 +729,13 @@ __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
     k_stream_collide_pair(LevelView v, float omega, RefF R, const __half* __restrict__ xf,
                           const __grid_constant__ EdgeArg<L> E) {
   if (edge_block<L, __half, COLL, PAR, MOV>(v, omega, R, E)) return;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x, y;
+  if constexpr (L::D == 3) {
+    plane_node(v, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y);
+  } else {
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+  }
   const int npairs = (v.batch + 1) / 2;
   int z = blockIdx.z - edge_slices(E), pair = 0;
   if (npairs > 1) {
@@ -674,8 +749,7 @@ __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
   const NodeAddr a = node_addr<L>(v, x, y, z);
   // a lane on a face normal to x takes its populations from the face buffer
   // (after the loads from the planes, in warps holding such a lane only)
-  const bool fw = warp_has_xface(v, xf);
-  const bool fx = fw && (x == 0 || x == v.n[0] - 1);
+  const bool fx = xf != nullptr && (x == 0 || x == v.n[0] - 1);
   F2 g[L::Q];  // lane x: run 2p, lane y: run 2p+1
   sfor<L::Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
@@ -687,7 +761,7 @@ __global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
     g[i].v = __half22float2(h);
   });
   if constexpr (L::D == 3) {  // (2D levels have no face buffer)
-    if (fw && fx) {
+    if (fx) {
       const long long F = (long long)v.n[1] * v.n[2];
       const __half2* xb = reinterpret_cast<const __half2*>(xf) +
                           ((long long)pair * 2 + (x != 0)) * L::Q * F + (long long)z * v.n[1] + y;

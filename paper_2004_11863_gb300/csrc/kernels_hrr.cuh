@@ -82,13 +82,18 @@ __global__ void k_velocity(LevelView v, float* du, int par, RefF ref) {
 }
 
 // ------------------------------------------------------ level update, H-RR
-// One thread per node, 32 x 4 blocks like the plain update.  ks = -2 tau
+// One thread per node, 128-thread blocks laid out like the plain update's.  ks = -2 tau
 // cs^2 (1 - sig) of this level.
 template <class L, class S, int PAR, bool MOV>
 __global__ void __launch_bounds__(128)
     k_stream_collide_hrr(LevelView v, float omega, RefF R, const float* du, float sig, float ks) {
-  const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * 4 + threadIdx.y;
+  int x, y;
+  if constexpr (L::D == 3) {
+    plane_node(v, blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x, x, y);
+  } else {
+    x = blockIdx.x * 32 + threadIdx.x;
+    y = blockIdx.y * 4 + threadIdx.y;
+  }
   int z = blockIdx.z, run = 0;
   if (v.batch > 1) {
     run = z / v.n[2];

@@ -394,10 +394,15 @@ int build_layout(lbm_ctx* h) {
   return LBM_OK;
 }
 
-// Storage geometry (ghost skin on bounded axes, row pitch a multiple of
-// MLBM_ROW_ALIGN elements).
+// Storage geometry (ghost skin on bounded axes).  Rows are padded to
+// MLBM_ROW_ALIGN elements in 2D; in 3D, whose updates walk the elements of a
+// plane (plane_node), to eight elements, with rows added until a plane is
+// whole 32-element lines -- unless that takes more memory than padded rows.
 #ifndef MLBM_ROW_ALIGN
 #define MLBM_ROW_ALIGN 32
+#endif
+#ifndef MLBM_ROW_ALIGN_3D
+#define MLBM_ROW_ALIGN_3D 8
 #endif
 void build_view(lbm_ctx* h, int l) {
   Level& v = h->lev[l];
@@ -406,6 +411,15 @@ void build_view(lbm_ctx* h, int l) {
   for (int a = 0; a < 3; ++a) g[a] = v.per[a] ? 0 : 1;
   w.SX = round_up(v.n[0] + 2 * g[0], MLBM_ROW_ALIGN);
   w.SY = v.n[1] + 2 * g[1];
+  if (h->D == 3) {
+    const int sx = round_up(v.n[0] + 2 * g[0], MLBM_ROW_ALIGN_3D);
+    const int lines = sx % 32 == 0 ? 1 : sx % 16 == 0 ? 2 : sx % 8 == 0 ? 4 : 8;
+    const int sy = round_up(w.SY, lines);
+    if ((long long)sx * sy <= (long long)w.SX * w.SY) {
+      w.SX = sx;
+      w.SY = sy;
+    }
+  }
   const long long SZ = v.n[2] + 2 * g[2];
   w.off = 32 + ((long long)g[2] * w.SY + g[1]) * w.SX;
   long long need = w.off + SZ * w.SY * (long long)w.SX + 32;
@@ -1023,6 +1037,10 @@ int lbm_create(const lbm_config* cfg, void* stream, const lbm_allocator* alloc,
     }
   }
   for (int l = 0; l < h->nlev; ++l) {
+    // blocks of one warp in 3D: a block's registers are held until its last
+    // warp has walked its planes (32 x 4 blocks: vortex3d 4.28 ms a step,
+    // 32 x 1 4.22; pulse3d 2.44 and 2.40; binary16 slab 885 and 860 us)
+    if (h->D == 3) h->lev[l].k1_by = 1;
     build_view(h, l);
     if (h->lev[l].view.plane > 2147483647LL) {  // kernels index planes in 32 bits
       delete h;

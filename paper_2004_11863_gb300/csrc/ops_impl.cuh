@@ -48,28 +48,44 @@ inline Edge2d with_slices(Edge2d E, int batch, dim3& grid, const dim3& block) {
   return E;
 }
 
+// Blocks of bx x by threads over one z-plane, `nodes` nodes per thread: 3D
+// along the plane's elements (plane_node), 2D rows.
+template <class L>
+dim3 plane_blocks(const LevelView& v, int bx, int by, int nodes) {
+  if (L::D == 3)
+    return dim3(blocks_for((long long)((v.n[1] + nodes - 1) / nodes - 1) * v.SX + v.n[0], bx * by));
+  return dim3((v.n[0] + bx - 1) / bx, (v.n[1] + by * nodes - 1) / (by * nodes));
+}
+
 template <class L, class S, int COLL>
 cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx,
                          int by, const S* xf, const EdgeArg<L>& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   if (v.run_stride >= (1LL << 31)) return cudaErrorInvalidValue;  // (32-bit offsets)
   dim3 block(bx, by, 1);
-  dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + 2 * by - 1) / (2 * by),
-            (v.n[2] + K1X2Pfz<S>::PZ - 1) / K1X2Pfz<S>::PZ * v.batch);
+  const dim3 xy = plane_blocks<L>(v, bx, by, 2);
+  dim3 grid(xy.x, xy.y,
+            (v.n[2] + K1X2Pfz<L, S>::PZ - 1) / K1X2Pfz<L, S>::PZ * v.batch);
   const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
-  if (mov) {
+  auto go = [&](auto M, auto X) {
+    constexpr bool MOV = decltype(M)::value, XF = decltype(X)::value;
     if (par == 0)
-      k_stream_collide_x2<L, S, COLL, 0, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
+      k_stream_collide_x2<L, S, COLL, 0, MOV, XF><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
-      k_stream_collide_x2<L, S, COLL, 1, true><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
-  } else {
-    if (par == 0)
-      k_stream_collide_x2<L, S, COLL, 0, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
-    else
-      k_stream_collide_x2<L, S, COLL, 1, false><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
-  }
+      k_stream_collide_x2<L, S, COLL, 1, MOV, XF><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
+  };
+  auto faces = [&](auto M) {
+    if constexpr (L::D == 3) {
+      if (xf != nullptr) return go(M, std::true_type{});
+    }
+    go(M, std::false_type{});
+  };
+  if (mov)
+    faces(std::true_type{});
+  else
+    faces(std::false_type{});
   return cudaGetLastError();
 }
 
@@ -107,7 +123,8 @@ cudaError_t sc_pair_launch(const LevelView& v, int par, float omega, const RefSt
                            int by, const __half* xf, const EdgeArg<L>& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   dim3 block(bx, by, 1);
-  dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + by - 1) / by, v.n[2] * ((v.batch + 1) / 2));
+  dim3 grid = plane_blocks<L>(v, bx, by, 1);
+  grid.z = v.n[2] * ((v.batch + 1) / 2);
   const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
@@ -313,7 +330,8 @@ template <class L, class S, bool MOV>
 void sc_hrr_t(const LevelView& v, int par, float omega, const float* du, float sig, float ks,
               const RefF& R, cudaStream_t s) {
   dim3 block(32, 4, 1);
-  dim3 grid((v.n[0] + 31) / 32, (v.n[1] + 3) / 4, v.n[2] * v.batch);
+  dim3 grid = plane_blocks<L>(v, 32, 4, 1);
+  grid.z = v.n[2] * v.batch;
   if (par == 0)
     k_stream_collide_hrr<L, S, 0, MOV><<<grid, block, 0, s>>>(v, omega, R, du, sig, ks);
   else
