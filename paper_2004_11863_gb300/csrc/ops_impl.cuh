@@ -464,11 +464,17 @@ cudaError_t macros_f(const LevelView& v, int storage, int run, int last, float* 
     R.m_hi[a] = (float)m;
     R.m_lo[a] = (float)(m - R.m_hi[a]);
   }
-  if (storage == 0)
-    k_macros_f<L, float><<<g, 128, 0, s>>>(v, run, last, rho, u, R);
-  else
-    k_macros_f<L, __half><<<g, 128, 0, s>>>(v, run, last, rho, u, R);
-  return cudaGetLastError();
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(g);
+  c.blockDim = dim3(128);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return storage == 0 ? cudaLaunchKernelEx(&c, k_macros_f<L, float>, v, run, last, rho, u, R)
+                      : cudaLaunchKernelEx(&c, k_macros_f<L, __half>, v, run, last, rho, u, R);
 }
 
 template <class L>
