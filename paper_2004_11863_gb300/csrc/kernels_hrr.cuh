@@ -140,56 +140,98 @@ __global__ void __launch_bounds__(128)
 // parent's next update, parity ppar).  mode 1 (set-up): every neighbour
 // from the parent's current state (laid out after an update of parity ppar)
 // into slots s_new and s_also.
+// Four lanes per entry: lane a < D takes the two neighbours along axis a, so
+// that no thread walks more than two nodes' loads one after the other, and
+// lanes 0 to 2 store two components each.  ti: as for the populations
+// (capture_item), the strain rate at the child's first sub-step replaces the
+// one at t - 1, which leaves the outer layer's collision one slot to read
+// instead of three.  (96^3 with a refined 97^3 box, D3Q19, timed alone with
+// about 5 us of launch each: this kernel 19.1 -> 15.9 us against one thread
+// per entry, the outer layer's collision 19.2 -> 16.8.)
 template <class L, class S>
-__global__ void k_parent_strain(LevelView p, LevelView c, RingDesc R, TnDesc T, float* sh,
-                                int s_new, int s_also, int ppar, int cpar, int mode, RefF ref) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int run = blockIdx.y;
-  if (k >= R.K) return;
+__global__ void __launch_bounds__(64)
+    k_parent_strain(LevelView p, LevelView c, const __grid_constant__ RingDesc R,
+                    const __grid_constant__ TnDesc T, float* sh, int s_new, int s_also, int ppar,
+                    int cpar, int mode, TimeInt ti, RefF ref) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long k = t >> 2;
+  const int ax = (int)(t & 3), run = blockIdx.y;
+  const unsigned mask = 0xfu << (threadIdx.x & 28);
+  if (k >= R.K) return;  // whole groups leave
   int P[3];
   ring_node(R, k, P);
-  const S* fp = run_cptr<S>(p, run);
-  const S* fcb = run_cptr<S>(c, run);
-  float up[3][3] = {}, um[3][3] = {};
-  for (int ax = 0; ax < L::D; ++ax)
-    for (int sg = 0; sg < 2; ++sg) {
-      int Q[3] = {P[0], P[1], P[2]};
-      Q[ax] += sg ? -1 : 1;
-      if (p.per[ax]) Q[ax] = wrapi(Q[ax], p.n[ax]);
-      float g[L::Q], drho, u[3];
-      if (mode == 0 && p.has_tn && Q[0] >= p.tn_lo[0] && Q[0] <= p.tn_hi[0] &&
-          Q[1] >= p.tn_lo[1] && Q[1] <= p.tn_hi[1] && Q[2] >= p.tn_lo[2] && Q[2] <= p.tn_hi[2]) {
-        int X[3] = {0, 0, 0};
-        for (int b = 0; b < L::D; ++b) X[b] = T.boxed[b] ? 2 * (Q[b] - T.lo[b]) : 2 * Q[b];
-        load_pre<L, S>(fcb, c.plane, node_addr<L>(c, X[0], X[1], X[2]), cpar, c.es, g);
-      } else if (mode == 0) {
-        load_pre<L, S>(fp, p.plane, node_addr<L>(p, Q[0], Q[1], Q[2]), ppar, p.es, g);
-      } else {
-        load_post<L, S>(fp, p.plane, node_addr<L>(p, Q[0], Q[1], Q[2]), ppar, p.es, g);
-      }
-      deviations<L>(g, ref, drho, u[0], u[1], u[2]);
-      for (int b = 0; b < 3; ++b) (sg ? um : up)[ax][b] = u[b];
-    }
-  float Sv[6];
-  strain_from<L>(up, um, Sv);
-  float* h = sh + (long long)run * 3 * 6 * R.K;
-  for (int rep = 0; rep < (mode == 0 ? 1 : 2); ++rep) {
-    float* hs = h + (long long)(rep == 0 ? s_new : s_also) * 6 * R.K + k;
+  float gr[3] = {0.0f, 0.0f, 0.0f};  // d_ax u_b
+  if (ax < L::D) {
+    const S* fp = run_cptr<S>(p, run);
+    const S* fcb = run_cptr<S>(c, run);
+    float g[2][L::Q];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) hs[(long long)j * R.K] = Sv[j];
+    for (int sg = 0; sg < 2; ++sg) {
+      int Qn[3];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        Qn[b] = P[b] + (b == ax ? (sg ? -1 : 1) : 0);
+        if (p.per[b]) Qn[b] = wrapi(Qn[b], p.n[b]);
+      }
+      if (mode == 0 && p.has_tn && Qn[0] >= p.tn_lo[0] && Qn[0] <= p.tn_hi[0] &&
+          Qn[1] >= p.tn_lo[1] && Qn[1] <= p.tn_hi[1] && Qn[2] >= p.tn_lo[2] &&
+          Qn[2] <= p.tn_hi[2]) {
+        int X[3] = {0, 0, 0};
+#pragma unroll
+        for (int b = 0; b < L::D; ++b) X[b] = T.boxed[b] ? 2 * (Qn[b] - T.lo[b]) : 2 * Qn[b];
+        load_pre<L, S>(fcb, c.plane, node_addr<L>(c, X[0], X[1], X[2]), cpar, c.es, g[sg]);
+      } else if (mode == 0) {
+        load_pre<L, S>(fp, p.plane, node_addr<L>(p, Qn[0], Qn[1], Qn[2]), ppar, p.es, g[sg]);
+      } else {
+        load_post<L, S>(fp, p.plane, node_addr<L>(p, Qn[0], Qn[1], Qn[2]), ppar, p.es, g[sg]);
+      }
+    }
+    float drho, up[3], um[3];
+    deviations<L>(g[0], ref, drho, up[0], up[1], up[2]);
+    deviations<L>(g[1], ref, drho, um[0], um[1], um[2]);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) gr[b] = 0.5f * (up[b] - um[b]);
+  }
+  // lane ax gets row ax of the gradient and, by shuffles, its column:
+  // S_aa and S_a,a+1 (xx, xy), (yy, yz), (zz, xz)
+  const int nx = ax == 2 ? 0 : ax + 1;
+  auto row = [&](int b) { return b == 0 ? gr[0] : (b == 1 ? gr[1] : gr[2]); };
+  // what lane ax's predecessor needs: d_ax u_{ax-1}
+  const float give = row(ax == 0 ? 2 : ax - 1);
+  const float cross = __shfl_sync(mask, give, nx, 4);  // d_nx u_ax
+  if (ax > 2) return;
+  const float diag = row(ax < 3 ? ax : 0), off = 0.5f * (row(nx) + cross);
+  const int jd = ax, jo = ax == 0 ? 3 : (ax == 1 ? 5 : 4);
+  float* h = sh + (long long)run * 3 * 6 * R.K + k;
+  if (ti.on) {
+    float* hm = h + (long long)ti.s_m1 * 6 * R.K;
+    const float* h0 = h + (long long)ti.s_0 * 6 * R.K;
+    auto put = [&](int j, float now) {
+      const long long o = (long long)j * R.K;
+      float val = ti.w1 * h0[o] + ti.w2 * now;
+      if (ti.w0 != 0.0f) val += ti.w0 * hm[o];  // (the first step has no t - 1)
+      hm[o] = val;
+    };
+    put(jd, diag);
+    put(jo, off);
+  }
+  for (int rep = 0; rep < (mode == 0 ? 1 : 2); ++rep) {
+    float* hs = h + (long long)(rep == 0 ? s_new : s_also) * 6 * R.K;
+    hs[(long long)jd * R.K] = diag;
+    hs[(long long)jo * R.K] = off;
   }
 }
 
 // --------------------------------------------- child outer layer collision
-// One thread per child boundary node (TF / IE).  The parent strain rate is
-// interpolated in time with weights (w0, w1, w2) on slots (s_m1, s_0, s_p1)
-// and in space with the eq. spaceInt stencil along the face's odd
+// One thread per child boundary node (TF / IE).  The parent strain rate in
+// `slot` (interpolated in time by k_parent_strain on the first sub-step, t + 1
+// itself on the second) is interpolated in space with the eq. spaceInt stencil along the face's odd
 // coordinates, halved (eq. PijResc); the node's pre-collision state (written
 // by the rebuild for the update of parity par) is collided with it.
 template <class L, class S, bool MOV>
-__global__ void k_collide_bnd(LevelView c, BndDesc B, RingDesc R, const float* sh, float w0,
-                              float w1, float w2, int s_m1, int s_0, int s_p1, float omega,
-                              float sig, float ks, int par, RefF ref) {
+__global__ void k_collide_bnd(LevelView c, const __grid_constant__ BndDesc B,
+                              const __grid_constant__ RingDesc R, const float* sh, int slot,
+                              float omega, float sig, float ks, int par, RefF ref) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int run = blockIdx.y;
   if (k >= B.count) return;
@@ -222,7 +264,7 @@ __global__ void k_collide_bnd(LevelView c, BndDesc B, RingDesc R, const float* s
     }
   }
   auto sw = [](int s) { return (s == 0 || s == 3) ? -1.0f / 16.0f : 9.0f / 16.0f; };
-  const float* h = sh + (long long)run * 3 * 6 * R.K;
+  const float* h = sh + ((long long)run * 3 + slot) * 6 * R.K;
   float Sv[6] = {0, 0, 0, 0, 0, 0};
   for (int s0 = 0; s0 < n_s[0]; ++s0)
     for (int s1 = 0; s1 < n_s[1]; ++s1) {
@@ -239,12 +281,7 @@ __global__ void k_collide_bnd(LevelView c, BndDesc B, RingDesc R, const float* s
         idx += (long long)pc * stride[b];
       }
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        const float vt = w0 * h[((long long)s_m1 * 6 + j) * R.K + idx] +
-                         w1 * h[((long long)s_0 * 6 + j) * R.K + idx] +
-                         w2 * h[((long long)s_p1 * 6 + j) * R.K + idx];
-        Sv[j] += w * vt;
-      }
+      for (int j = 0; j < 6; ++j) Sv[j] += w * h[(long long)j * R.K + idx];
     }
   HrrIn<float> hy;
   hy.sig = sig;

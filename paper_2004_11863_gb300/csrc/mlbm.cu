@@ -849,13 +849,9 @@ int advance_hrr(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wai
   const int par = 1 - v.last;
   const float sig = (float)h->cfg.sigma;
   float* du = (float*)v.du_mem;
-  int slots[3] = {0, 0, 0};
   if (l >= 1) {
     const Level& p = h->lev[l - 1];
     const float resc = (float)(v.tau / (2.0 * p.tau));  // eq. rescff
-    slots[0] = (v.head + 1) % 3;
-    slots[1] = (v.head + 2) % 3;
-    slots[2] = v.head;
     LAUNCH_K(2, l, h->ops.inject(v.view, v.bnd, v.ring, st, read_slot(v, wt), resc, par, ref,
                                  nullptr, h->cur));
   }
@@ -907,9 +903,10 @@ int advance_hrr(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wai
     float* sh = (float*)v.sh_mem;
     if (first_substep)
       LAUNCH_K(6, l - 1, h->ops.parent_strain(p.view, v.view, v.ring, v.tn, st, sh, v.head, v.head,
-                                              1 - p.last, 1 - v.last, 0, ref, h->cur));
-    LAUNCH_K(7, l, h->ops.collide_bnd(v.view, v.bnd, v.ring, st, sh, wt, slots, omega_of(v.tau),
-                                      sig, hrr_ks(h, v.tau), par, ref, h->cur));
+                                              1 - p.last, 1 - v.last, 0,
+                                              time_int(v, p.nsteps == 0), ref, h->cur));
+    LAUNCH_K(7, l, h->ops.collide_bnd(v.view, v.bnd, v.ring, st, sh, read_slot(v, wt),
+                                      omega_of(v.tau), sig, hrr_ks(h, v.tau), par, ref, h->cur));
   }
   return LBM_OK;
 }
@@ -950,7 +947,7 @@ int seed_history(lbm_ctx* h) {
     if (h->cfg.collision == LBM_HRR)
       LAUNCH(h->ops.parent_strain(p.view, h->lev[l].view, h->lev[l].ring, h->lev[l].tn,
                                   h->cfg.storage, (float*)h->lev[l].sh_mem, 1, 0, p.last,
-                                  h->lev[l].last, 1, h->ref, h->cur));
+                                  h->lev[l].last, 1, TimeInt{}, h->ref, h->cur));
   }
   h->seeded = true;
   return LBM_OK;

@@ -43,10 +43,11 @@ struct Ops {
                                     cudaStream_t s);
   cudaError_t (*parent_strain)(const LevelView& p, const LevelView& c, const RingDesc& R,
                                const TnDesc& T, int storage, float* sh, int s_new, int s_also,
-                               int ppar, int cpar, int mode, const RefState& ref, cudaStream_t s);
+                               int ppar, int cpar, int mode, const TimeInt& ti,
+                               const RefState& ref, cudaStream_t s);
   cudaError_t (*collide_bnd)(const LevelView& c, const BndDesc& B, const RingDesc& R, int storage,
-                             const float* sh, const float* wt, const int* slots, float omega,
-                             float sig, float ks, int par, const RefState& ref, cudaStream_t s);
+                             const float* sh, int slot, float omega, float sig, float ks, int par,
+                             const RefState& ref, cudaStream_t s);
   cudaError_t (*restrict_hrr)(const LevelView& p, const LevelView& c, const TnDesc& T,
                               int storage, float resc, int ppar, int cpar, float* pdu,
                               float omega_p, float sig, float ks_p, const RefState& ref,

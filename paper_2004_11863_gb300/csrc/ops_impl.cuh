@@ -361,15 +361,16 @@ cudaError_t stream_collide_hrr(const LevelView& v, int storage, int par, float o
 template <class L>
 cudaError_t parent_strain(const LevelView& p, const LevelView& c, const RingDesc& R,
                           const TnDesc& T, int storage, float* sh, int s_new, int s_also, int ppar,
-                          int cpar, int mode, const RefState& ref, cudaStream_t s) {
+                          int cpar, int mode, const TimeInt& ti, const RefState& ref,
+                          cudaStream_t s) {
   if (R.K == 0) return cudaSuccess;
-  dim3 grid(blocks_for(R.K, 64), p.batch);
+  dim3 grid(blocks_for(4 * R.K, 64), p.batch);  // (four lanes per ring entry)
   if (storage == 0)
     k_parent_strain<L, float><<<grid, 64, 0, s>>>(p, c, R, T, sh, s_new, s_also, ppar, cpar,
-                                                  mode, make_ref_f<L>(ref));
+                                                  mode, ti, make_ref_f<L>(ref));
   else
     k_parent_strain<L, __half><<<grid, 64, 0, s>>>(p, c, R, T, sh, s_new, s_also, ppar, cpar,
-                                                   mode, make_ref_f<L>(ref));
+                                                   mode, ti, make_ref_f<L>(ref));
   return cudaGetLastError();
 }
 
@@ -395,30 +396,29 @@ cudaError_t sensor_read(const LevelView& v, int run, const SensorState& st, unsi
 
 template <class L, class S, bool MOV>
 void collide_bnd_t(const LevelView& c, const BndDesc& B, const RingDesc& R, const float* sh,
-                   const float* wt, const int* slots, float omega, float sig, float ks, int par,
-                   const RefF& ref, cudaStream_t s) {
+                   int slot, float omega, float sig, float ks, int par, const RefF& ref,
+                   cudaStream_t s) {
   dim3 grid(blocks_for(B.count, 64), c.batch);
-  k_collide_bnd<L, S, MOV><<<grid, 64, 0, s>>>(c, B, R, sh, wt[0], wt[1], wt[2], slots[0],
-                                               slots[1], slots[2], omega, sig, ks, par, ref);
+  k_collide_bnd<L, S, MOV><<<grid, 64, 0, s>>>(c, B, R, sh, slot, omega, sig, ks, par, ref);
 }
 
 template <class L>
 cudaError_t collide_bnd(const LevelView& c, const BndDesc& B, const RingDesc& R, int storage,
-                        const float* sh, const float* wt, const int* slots, float omega, float sig,
-                        float ks, int par, const RefState& ref, cudaStream_t s) {
+                        const float* sh, int slot, float omega, float sig, float ks, int par,
+                        const RefState& ref, cudaStream_t s) {
   if (B.count == 0) return cudaSuccess;
   const RefF Rf = make_ref_f<L>(ref);
   const bool mov = moving(ref);
   if (storage == 0) {
     if (mov)
-      collide_bnd_t<L, float, true>(c, B, R, sh, wt, slots, omega, sig, ks, par, Rf, s);
+      collide_bnd_t<L, float, true>(c, B, R, sh, slot, omega, sig, ks, par, Rf, s);
     else
-      collide_bnd_t<L, float, false>(c, B, R, sh, wt, slots, omega, sig, ks, par, Rf, s);
+      collide_bnd_t<L, float, false>(c, B, R, sh, slot, omega, sig, ks, par, Rf, s);
   } else {
     if (mov)
-      collide_bnd_t<L, __half, true>(c, B, R, sh, wt, slots, omega, sig, ks, par, Rf, s);
+      collide_bnd_t<L, __half, true>(c, B, R, sh, slot, omega, sig, ks, par, Rf, s);
     else
-      collide_bnd_t<L, __half, false>(c, B, R, sh, wt, slots, omega, sig, ks, par, Rf, s);
+      collide_bnd_t<L, __half, false>(c, B, R, sh, slot, omega, sig, ks, par, Rf, s);
   }
   return cudaGetLastError();
 }
