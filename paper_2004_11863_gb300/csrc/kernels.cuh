@@ -1103,28 +1103,32 @@ __global__ void __launch_bounds__(InjSep<L>::NT)
   const long long K = R.K;
   const float* h = R.hist + ((long long)run * 3 + slot) * R.nv * K;
   const int tid = threadIdx.y * T::TI + threadIdx.x;
-  // stage
-#pragma unroll(T::UNR)
-  for (int e = tid; e < T::NV * T::WJ * T::WI; e += T::NT) {
-    const int pi = e % T::WI, pj = (e / T::WI) % T::WJ, vv = e / (T::WI * T::WJ);
+  // ring entry of every window node (once per node, not once per value)
+  __shared__ int ring[T::WJ * T::WI];
+  for (int e = tid; e < T::WJ * T::WI; e += T::NT) {
+    const int pi = e % T::WI, pj = e / T::WI;
     int ri = p0i + pi, rj = p0j + pj;
     bool ok = true;
-    long long idx = R.start[f];
     if (bx1) {
-      ok = ok && ri >= -1 && ri <= e1 - 2;
-      idx += (long long)(ri + 1) * st1;
+      ok = ri >= -1 && ri <= e1 - 2;
+      ri += 1;
     } else {
       ri = ((ri % pn1) + pn1) % pn1;
-      idx += (long long)ri * st1;
     }
     if (bx2) {
       ok = ok && rj >= -1 && rj <= e2 - 2;
-      idx += (long long)(rj + 1) * st2;
+      rj += 1;
     } else {
       rj = ((rj % pn2) + pn2) % pn2;
-      idx += (long long)rj * st2;
     }
-    sv[vv][pj][pi] = ok ? h[vv * K + idx] : 0.0f;
+    ring[e] = ok ? (int)(R.start[f] + ri * st1 + rj * st2) : -1;
+  }
+  __syncthreads();
+  // stage
+#pragma unroll(T::UNR)
+  for (int e = tid; e < T::NV * T::WJ * T::WI; e += T::NT) {
+    const int vv = e / (T::WI * T::WJ), idx = ring[e - vv * (T::WI * T::WJ)];
+    (&sv[0][0][0])[e] = idx >= 0 ? h[vv * K + idx] : 0.0f;
   }
   __syncthreads();
   // along t1 (eq. spaceInt weights -1/16, 9/16, 9/16, -1/16 at odd child
