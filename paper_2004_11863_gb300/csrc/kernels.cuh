@@ -3,13 +3,15 @@
 //   k_stream_collide  fused stream + collide of every active node of a level
 //                     (eq. LBMequation), in place with the AA pattern;
 //   k_capture         parent pre-collision (drho, u, f^(1)) at t+1 on a child
-//                     box surface -> three-slot history;
-//   k_inject          child TF / IE nodes: temporal (eq. TempInt) and spatial
-//                     (eq. spaceInt) interpolation staged per face tile in
-//                     shared memory, rescaling (eq. rescff), written where
-//                     the child's next update reads them (2D; k_inject_sep,
-//                     the same with the stencil applied one axis at a time,
-//                     in 3D);
+//                     box surface -> three-slot history (its first sub-step's state interpolated in time, eq.
+//                     TempInt);
+//   k_inject          child TF / IE nodes: spatial (eq. spaceInt)
+//                     interpolation staged per face tile in shared memory,
+//                     rescaling (eq. rescff), written where the child's next
+//                     update reads them (2D with sensors or the hybrid
+//                     collision; k_inject_sep, the same with the stencil
+//                     applied one axis at a time, in 3D; other 2D updates
+//                     take these nodes along, kernels_edge.cuh);
 //   k_restrict_tile   parent TN nodes: filtered child f^(1) (eq. filterFneq),
 //                     rescaling (eq. rescfc), written where the parent's next
 //                     update reads them (the restriction), per face tile; with
@@ -529,8 +531,8 @@ struct K1X2Tune<D3Q27> {
 // nested case, +7 % on a 161 x 97 x 83 level; two, -1 %); binary16: 1 (its
 // update is nearer the instruction limit: with four planes the slab's step
 // takes 937 us, not 860).  Measured on GB300.
-#ifndef K1X2_PFZ_19F
-#define K1X2_PFZ_19F 8
+#ifndef K1X2_PFZ_F
+#define K1X2_PFZ_F 8
 #endif
 #ifndef K1X2_PFZ_27F
 #define K1X2_PFZ_27F 4
@@ -542,7 +544,7 @@ template <class L, class S>
 struct K1X2Pfz {
   static constexpr int PZ = !std::is_same<S, float>::value ? K1X2_PFZ_H
                             : L::Q == 27                   ? K1X2_PFZ_27F
-                                                           : K1X2_PFZ_19F;
+                                                           : K1X2_PFZ_F;
 };
 
 // Node (x, y) at element e of a 3D level's z-plane, counted from its first
@@ -698,6 +700,66 @@ __global__ void __launch_bounds__(128, !std::is_same<S, float>::value
       stream_collide_x2_pair<L, S, COLL, PAR, MOV, XF>(v, omega, R, xf, E, x, y0, z, run);
     }
   }
+}
+
+// Even update of a 3D level in binary16 (es = 1): the nodes (x, x + 1), x
+// even, take the two lanes, so each direction of both moves with one 4-byte
+// access -- an even update touches no shifted cell -- in place of two 2-byte
+// ones, and waits in one register instead of two: the update is bound by the
+// loads its warps can keep in flight.  (Fine level of a 160^3 slab, both
+// parities together 314 -> 288 us an update, step 833 -> 788; five blocks per
+// SM, six 807, four 818.  BGK keeps the populations to the end: one fewer.)
+#ifndef K1EH_MINB_D3Q19
+#define K1EH_MINB_D3Q19 5
+#endif
+#ifndef K1EH_MINB_D3Q27
+#define K1EH_MINB_D3Q27 4
+#endif
+template <class L, int COLL, bool MOV, bool XF>
+__global__ void __launch_bounds__(128, (L::Q == 27 ? K1EH_MINB_D3Q27 : K1EH_MINB_D3Q19) -
+                                           (COLL == 0 ? 1 : 0))
+    k_stream_collide_even_h(LevelView v, float omega, RefF R, const __half* __restrict__ xf) {
+  const unsigned e = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+  const unsigned hx = (unsigned)v.SX / 2, row = e / hx;
+  const int x = 2 * (int)(e - row * hx), y = (int)row;
+  int z = blockIdx.z, run = 0;
+  if (v.batch > 1) {
+    run = z / v.n[2];
+    z -= run * v.n[2];
+  }
+  if (x >= v.n[0] || y >= v.n[1]) return;
+  const bool ok0 = !inactive(v, x, y, z), ok1 = x + 1 < v.n[0] && !inactive(v, x + 1, y, z);
+  if (!ok0 && !ok1) return;
+  __half2* f = reinterpret_cast<__half2*>(static_cast<__half*>(v.f) + run * v.run_stride);
+  const int ph = (int)(v.plane / 2), at = ((int)v.off + (z * v.SY + y) * v.SX + x) / 2;
+  __half2 h[L::Q];
+  sfor<L::Q>([&](auto I) { h[decltype(I)::value] = f[decltype(I)::value * ph + at]; });
+  if constexpr (XF) {
+    // nodes on the faces normal to x: from the face buffer
+    const bool f0 = x == 0 || x == v.n[0] - 1, f1 = x + 1 == v.n[0] - 1;
+    if (f0 || f1) {
+      const long long F = (long long)v.n[1] * v.n[2];
+      const __half* xb =
+          xf + ((long long)run * 2 + (x != 0)) * L::Q * F + (long long)z * v.n[1] + y;
+      sfor<L::Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        const __half b = xb[i * F];
+        h[i] = f0 ? __halves2half2(b, __high2half(h[i])) : __halves2half2(__low2half(h[i]), b);
+      });
+    }
+  }
+  F2 g[L::Q];
+  sfor<L::Q>([&](auto I) { g[decltype(I)::value].v = __half22float2(h[decltype(I)::value]); });
+  collide_emit<L, COLL, MOV>(g, omega, R, [&](auto I, F2 val) {
+    const __half2 o = __float22half2_rn(val.v);
+    __half2* p = &f[opp<L>(decltype(I)::value) * ph + at];
+    if (ok0 && ok1)
+      *p = o;
+    else if (ok0)
+      *reinterpret_cast<__half*>(p) = __low2half(o);
+    else
+      *(reinterpret_cast<__half*>(p) + 1) = __high2half(o);
+  });
 }
 
 // Level update of binary16 storage with runs interleaved in pairs (es = 2):

@@ -16,6 +16,8 @@
 // The coarse level therefore streams and collides in one fused pass after
 // the fine sub-steps: nothing it streams is changed by the fine sub-steps
 // except its TN nodes, which the restriction rebuilds anyway.
+// In 2D the updates rebuild their own special nodes (kernels_edge.cuh): a step
+// is capture, advance(l+1), K1, advance(l+1), without K3 and K4.
 #include <cuda_runtime.h>
 
 #include <algorithm>

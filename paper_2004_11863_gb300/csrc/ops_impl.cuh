@@ -71,6 +71,15 @@ cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefStat
   const RefF R = make_ref_f<L>(ref);
   auto go = [&](auto M, auto X) {
     constexpr bool MOV = decltype(M)::value, XF = decltype(X)::value;
+    if constexpr (L::D == 3 && std::is_same<S, __half>::value) {
+      // (rows, planes and runs of these levels start on even elements)
+      if (par == 0 && v.es == 1 && v.SX % 2 == 0 && v.off % 2 == 0 && v.plane % 2 == 0) {
+        const long long pairs = (long long)(v.n[1] - 1) * (v.SX / 2) + (v.n[0] + 1) / 2;
+        const dim3 eg(blocks_for(pairs, bx * by), 1, v.n[2] * v.batch);
+        k_stream_collide_even_h<L, COLL, MOV, XF><<<eg, block, 0, s>>>(v, omega, R, xf);
+        return;
+      }
+    }
     if (par == 0)
       k_stream_collide_x2<L, S, COLL, 0, MOV, XF><<<grid, block, 0, s>>>(v, omega, R, xf, Eg);
     else
