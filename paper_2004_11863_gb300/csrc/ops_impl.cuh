@@ -108,6 +108,10 @@ cudaError_t sc_launch(const LevelView& v, int par, float omega, const RefState& 
     if (v.run_stride < (1LL << 31)) return sc_x2_launch<L, S, COLL>(v, par, omega, ref, bx, by, xf, E, s);
   constexpr int NPT = K1Tune<L, S>::NPT;
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
+  if (v.n[1] > 65535 * by * NPT) {  // (this kernel's grid has a row of blocks per by rows)
+    bx = 32;
+    by = 4;
+  }
   dim3 block(bx, by, 1);
   dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + by * NPT - 1) / (by * NPT), v.n[2] * v.batch);
   const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
