@@ -292,11 +292,10 @@ struct StripAddr {
 //   ((((r / es) * 2 + s) * q + i) * F + z * n[1] + y) * es + r % es,
 // F = n[1] * n[2].  (3D levels only: a 2D face holds n[1] nodes of q = 9
 // populations, where the scattered stores cost little.)  The level update
-// reads a face node's populations from
-// here; a warp holds such a node only if it covers x = 0 or x = n[0] - 1,
-// and only those warps load from the face buffer (a warp-uniform branch
-// after the loads every lane issues from the planes, so that the other
-// warps run the same code as without face buffers).
+// reads a face node's populations from here: the two-node update in the one
+// load of the warps that hold such a node (stream_collide_x2_pair), the
+// one-node update of the largest runs and the paired one after the loads
+// that every lane issues from the planes, in those warps only.
 __device__ __forceinline__ bool warp_has_xface(const LevelView& v, const void* xf) {
   const int xw = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   return xf != nullptr && (xw == 0 || (xw <= v.n[0] - 1 && v.n[0] - 1 < xw + 32));

@@ -213,7 +213,8 @@ __host__ __device__ __forceinline__ void third_coeffs(T ux, T uy, T uz, T dux, T
   dA[XYZ] = dux * uy * uz + Ux * (duy * uz + Uy * duz);
 }
 
-// Equilibrium deviation for direction I:
+// Equilibrium deviation for direction I (FP64: the reference's own values, on
+// the host and in the population read-out; the steps use expand below):
 //   g0_i = f0_i(rho0 + drho, U + du) - f0_i(rho0, U)
 //        = w_i [ drho (1 + e_i(u)) + rho0 (e_i(u) - e_i(U)) ],
 //   e_i(u) = 3 xi.u + 4.5 (xi.u)^2 - 1.5 u.u + T3_i(u u u),
