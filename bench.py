@@ -61,15 +61,14 @@ NCU_TRAFFIC = {
 
 
 def kernel_source_hash() -> str:
-    """Hash of the level update's source: lattice.cuh and lattice_x2.cuh
-    (the collisions) and the part of kernels.cuh from the addressing helpers
-    to the end of the paired binary16 update.  Edits elsewhere do not void a
+    """Hash of the level update's source: lattice.cuh (the collisions) and
+    the part of kernels.cuh from the addressing helpers to the end of the
+    paired binary16 update.  Edits elsewhere do not void a
     traffic capture."""
     csrc = os.path.join(ROOT, "paper_2004_11863_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("lattice.cuh", "lattice_x2.cuh"):
-        with open(os.path.join(csrc, f), "rb") as fh:
-            h.update(fh.read())
+    with open(os.path.join(csrc, "lattice.cuh"), "rb") as fh:
+        h.update(fh.read())
     with open(os.path.join(csrc, "kernels.cuh"), "r") as fh:
         k = fh.read()
     start = k.index("__device__ __forceinline__ int wrapi")
