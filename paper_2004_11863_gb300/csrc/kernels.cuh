@@ -779,21 +779,26 @@ struct K1PairTune;
 #ifndef K1P_MINB_D3Q27
 #define K1P_MINB_D3Q27 3
 #endif
+// (the regularized collisions need 126 to 138 registers on D3Q27, and pass
+// 128 or not with small changes: bound there, four blocks an SM)
+#ifndef K1P_MINB_REG_D3Q27
+#define K1P_MINB_REG_D3Q27 4
+#endif
 template <>
 struct K1PairTune<D2Q9> {
-  static constexpr int MINB = K1P_MINB_D2Q9;
+  static constexpr int MINB = K1P_MINB_D2Q9, MINB_REG = MINB;
 };
 template <>
 struct K1PairTune<D3Q19> {
-  static constexpr int MINB = K1P_MINB_D3Q19;
+  static constexpr int MINB = K1P_MINB_D3Q19, MINB_REG = MINB;
 };
 template <>
 struct K1PairTune<D3Q27> {
-  static constexpr int MINB = K1P_MINB_D3Q27;
+  static constexpr int MINB = K1P_MINB_D3Q27, MINB_REG = K1P_MINB_REG_D3Q27;
 };
 
 template <class L, int COLL, int PAR, bool MOV>
-__global__ void __launch_bounds__(128, K1PairTune<L>::MINB)
+__global__ void __launch_bounds__(128, COLL == 0 ? K1PairTune<L>::MINB : K1PairTune<L>::MINB_REG)
     k_stream_collide_pair(LevelView v, float omega, RefF R, const __half* __restrict__ xf,
                           const __grid_constant__ EdgeArg<L> E) {
   if (edge_block<L, __half, COLL, PAR, MOV>(v, omega, R, E)) return;
