@@ -367,7 +367,9 @@ int lbm_profile(lbm_handle h, int enable);
  * kind (0 level update, 1 history capture, 2 coarse-to-fine rebuild,
  * 3 fine-to-coarse restriction, 4 probe sampling, 5 velocity pass (LBM_HRR
  * or sensors), 6 parent strain-rate history and 7 outer-layer collision
- * (LBM_HRR), 8 sensor pass) on one level
+ * (LBM_HRR), 8 sensor pass) on one level; in 2D without LBM_HRR 2 counts the
+ * launches that rebuild and collide the nodes of 2 and 3 in one go, and none
+ * where the update's launch (0) does so
  * (-1: all levels; the level is the one updated, or the parent for 1, 3
  * and 6).
  * Synchronises. */

@@ -166,13 +166,16 @@ struct TimeInt {
   float w0, w1, w2;
 };
 
-// Special nodes of a 2D level update, rebuilt and collided by blocks of their
-// own in the update's launch (kernels_edge.cuh).  Up to four faces.
-struct Edge2d {
-  int nz;        // leading z-slices of the grid that hold these blocks (0: none)
-  int wide;      // several lanes per node
-  int nb, nt;    // rebuilt outer nodes and TN nodes per run (0: the update's own blocks
-                 // take them like any other node)
+// Special nodes of a 2D level per run: rebuilt outer nodes and TN nodes (0: the
+// level has none, or an update takes them like any other node).
+struct EdgeCount {
+  int nb, nt;
+};
+
+// Special nodes of a 2D level update, rebuilt and collided by threads of their
+// own (kernels_edge.cuh).  Up to four faces.
+struct Edge2d : EdgeCount {
+  int nz;        // leading z-slices of the update's grid that hold their blocks
   int nf;        // faces of the level's own box
   int b_start[5], b_axis[4], b_side[4], b_lo[4];  // outer nodes by face, along its tangent
   int r_start[4];       // history-ring offset of each face
@@ -188,6 +191,16 @@ struct Edge2d {
   int cpar;             // parity of the child's next update
   float t_resc;         // eq. rescfc
 };
+
+// Whether the special nodes of a launch of `batch` runs are few
+// (kernels_edge.cuh): the lanes they take, four an outer node and sixteen a TN
+// node, up to about what the GPU holds beside an update's blocks.
+#ifndef EDGE_WIDE_LANES
+#define EDGE_WIDE_LANES 65536
+#endif
+inline bool edges_few(const EdgeCount& E, int batch) {
+  return (4LL * E.nb + 16LL * E.nt) * batch <= EDGE_WIDE_LANES;
+}
 
 // Persistent fused step (kernels_fused.cuh): the recorded program, the
 // launch arguments and the host-side description of the tables it reads.

@@ -8,14 +8,16 @@
 //   k_inject          child TF / IE nodes: spatial (eq. spaceInt)
 //                     interpolation staged per face tile in shared memory,
 //                     rescaling (eq. rescff), written where the child's next
-//                     update reads them (2D with sensors or the hybrid
-//                     collision; k_inject_sep, the same with the stencil
-//                     applied one axis at a time, in 3D; other 2D updates
-//                     take these nodes along, kernels_edge.cuh);
+//                     update reads them (2D with the hybrid collision;
+//                     k_inject_sep, the same with the stencil applied one
+//                     axis at a time, in 3D);
 //   k_restrict_tile   parent TN nodes: filtered child f^(1) (eq. filterFneq),
 //                     rescaling (eq. rescfc), written where the parent's next
-//                     update reads them (the restriction), per face tile; with
-//                     the hybrid collision it also collides the TN nodes;
+//                     update reads them (the restriction), per face tile (3D
+//                     and the hybrid collision, where it also collides them);
+//   k_edges           both kinds of node in 2D, rebuilt, collided and stored in
+//                     one go, unless the update's own launch does it
+//                     (kernels_edge.cuh);
 //   k_init / k_macros / k_diag_* / k_probe   set-up and read-out.
 //
 // AA pattern.  A step of parity 0 reads g_i of node n from plane i at n and
@@ -306,12 +308,12 @@ __device__ __forceinline__ bool warp_has_xface(const LevelView& v, const void* x
 // before the first collision.  The block shape (blockDim.x a multiple of 32,
 // blockDim.x * blockDim.y <= 128) is chosen at run time (lbm_autotune); it
 // changes which nodes share a block, not any node's arithmetic.
-template <class L, int COLL, class S, int PAR, bool MOV>
+template <class L, int COLL, class S, int PAR, bool MOV, class EG>
 __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
                                            : (PAR == 0 ? K1Tune<L, S>::MINB_EVEN
                                                        : K1Tune<L, S>::MINB))
     k_stream_collide(LevelView v, float omega, RefF R, const S* __restrict__ xf,
-                     const __grid_constant__ EdgeArg<L> E) {
+                     const __grid_constant__ EG E) {
   constexpr int NPT = K1Tune<L, S>::NPT;
   if (edge_block<L, S, COLL, PAR, MOV>(v, omega, R, E)) return;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -578,10 +580,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 }
 
 // XF: the level has a face buffer, xf.
-template <class L, class S, int COLL, int PAR, bool MOV, bool XF>
+template <class L, class S, int COLL, int PAR, bool MOV, bool XF, class EG>
 __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float omega,
                                                        const RefF& R, const S* __restrict__ xf,
-                                                       const EdgeArg<L>& E, int x, int y0, int z,
+                                                       const EG& E, int x, int y0, int z,
                                                        int run) {
   const bool ok0 = y0 < v.n[1] && !inactive(v, x, y0, z) && !edge_node(v, E, x, y0);
   const bool ok1 = y0 + 1 < v.n[1] && !inactive(v, x, y0 + 1, z) && !edge_node(v, E, x, y0 + 1);
@@ -643,7 +645,7 @@ __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float
   });
 }
 
-template <class L, class S, int COLL, int PAR, bool MOV, bool XF>
+template <class L, class S, int COLL, int PAR, bool MOV, bool XF, class EG>
 __global__ void __launch_bounds__(128, !std::is_same<S, float>::value
                                            ? (PAR ? K1X2Tune<L>::MINB1_H : K1X2Tune<L>::MINB_H)
                                        : PAR == 0  ? K1X2Tune<L>::MINB
@@ -651,7 +653,7 @@ __global__ void __launch_bounds__(128, !std::is_same<S, float>::value
                                        : XF        ? K1X2Tune<L>::MINB1_XF
                                                    : K1X2Tune<L>::MINB1)
     k_stream_collide_x2(LevelView v, float omega, RefF R, const S* __restrict__ xf,
-                        const __grid_constant__ EdgeArg<L> E) {
+                        const __grid_constant__ EG E) {
   constexpr int PZ = K1X2Pfz<L, S>::PZ;
   if (edge_block<L, S, COLL, PAR, MOV>(v, omega, R, E)) return;
   const int nzb = (v.n[2] + PZ - 1) / PZ;  // z blocks per run
@@ -797,10 +799,10 @@ struct K1PairTune<D3Q27> {
   static constexpr int MINB = K1P_MINB_D3Q27, MINB_REG = K1P_MINB_REG_D3Q27;
 };
 
-template <class L, int COLL, int PAR, bool MOV>
+template <class L, int COLL, int PAR, bool MOV, class EG>
 __global__ void __launch_bounds__(128, COLL == 0 ? K1PairTune<L>::MINB : K1PairTune<L>::MINB_REG)
     k_stream_collide_pair(LevelView v, float omega, RefF R, const __half* __restrict__ xf,
-                          const __grid_constant__ EdgeArg<L> E) {
+                          const __grid_constant__ EG E) {
   if (edge_block<L, __half, COLL, PAR, MOV>(v, omega, R, E)) return;
   int x, y;
   if constexpr (L::D == 3) {

@@ -1,44 +1,57 @@
 // Special nodes of a 2D level update: the outer nodes a level rebuilds from
 // its parent (eqs. spaceInt, rescff) and the TN nodes it takes from its child
-// (eqs. filterFneq, rescfc), rebuilt, collided and stored here in one go, in
-// blocks of the level update's own launch.
+// (eqs. filterFneq, rescfc), rebuilt, collided and stored here in one go.
 //
 // In the AA pattern a node's update reads and writes only the node's own
 // cells, so these nodes need no order against the rest of their level: a
 // coarse step of a 2D run is a chain of one capture and the level updates,
-// without a rebuild before every update, a restriction beside it, and the
-// stream forks that ran them side by side.  A small run is bound by the
-// latency of that chain (a kernel of a few blocks costs about two
-// microseconds whatever it does), a large one saves the pass of the rebuilt
-// populations through memory.
-// A run with few special nodes (E.wide: a chain of small launches) spreads a
-// node over lanes -- four for an outer node, one per tap of its stencil,
+// without a rebuild before every update and a restriction beside it.
+//
+// Few of them (edges_few) go into leading blocks of the update's own launch: a
+// small run is bound by the latency of its chain of launches (a kernel of a
+// few blocks costs about two microseconds whatever it does).  A node is then
+// spread over lanes -- four for an outer node, one per tap of its stencil,
 // sixteen for a TN node, one per child under the filter -- that exchange sums
-// by shuffles, so that no lane walks dependent loads; with many (a large
-// batch) a lane takes a whole node, which issues a fourth of the
-// instructions.  The sums are formed in the same order either way.
+// by shuffles, so that no lane walks dependent loads.  Many of them (a large
+// batch) go into a launch of their own beside the update's, one lane a node,
+// which issues a fourth of the instructions: compiled into the update that
+// path sets its registers (binary32 update 40 and 160 to 208 bytes of spills,
+// now 39 to 40 and none; 33 runs of 512^2 + 513^2 354 -> 333 us a step, 1024 of
+// 128 x 64 with a refined slab 924 -> 855).  The sums are formed in the same
+// order either way.
 // Per coarse step, against a rebuild before every update and a restriction
-// on a second stream: 128 x 64 run with a refined slab 19.7 -> 12.4 us (22.6
-// with one lane per node), 592^2 binary16 run of three levels 59.2 -> 43.6;
-// 33 runs of 512^2 + 513^2 327 -> 332 us in binary32, 207 -> 202 in binary16
-// (one lane per node; 357 and 219 with several).
+// on a second stream: the 128 x 64 run 20.4 -> 11.3 us, 592^2 binary16 run of
+// three levels 68 -> 43, 33 runs of 512^2 + 513^2 362 -> 333 in binary32,
+// 247 -> 203 in binary16.
+// The line between the two (lanes of the fine and of the coarse level's
+// launch; us a step within the update, beside it with one lane a node, beside
+// it with several): 512^2 + 513^2, 1 run (8 k, 16 k) 18.6, 20.9, 17.9; 4 runs
+// (33 k, 65 k) 40.9, 40.2, 42.0; 8 runs (66 k, 131 k) 84.1, 82.1, 85.2; 12 runs
+// (98 k, 197 k) 130.8, 127.2, 132.2; 128 x 64, 8 runs (8 k, 16 k) 14.9, 20.7,
+// 17.1; 64 runs (66 k, 131 k) 40.2, 41.6, 42.1.
+//
+// Levels with sensors, whose velocity pass needs the special nodes' velocity
+// before the update, take a launch of their own for any number, which writes
+// it (512^2 + 513^2, sensors on level 0: 38 -> 28 us a step against a rebuild
+// into the planes before it and a second one in the update).
 #pragma once
 
+// What an update kernel is told of them: nothing (3D, and 2D levels without
+// any), the nodes it leaves alone (EdgeCount), or those its own leading blocks
+// take (Edge2d).
 template <class L>
 struct NoEdge {};
-template <class L>
-using EdgeArg = std::conditional_t<L::D == 2, Edge2d, NoEdge<L>>;
 
-template <class L>
-__device__ __forceinline__ int edge_slices(const NoEdge<L>&) { return 0; }
+template <class E>
+__device__ __forceinline__ int edge_slices(const E&) { return 0; }
 __device__ __forceinline__ int edge_slices(const Edge2d& E) { return E.nz; }
 
-// Nodes the special blocks of the launch take.
+// Nodes that other threads take.
 template <class L>
 __device__ __forceinline__ bool edge_node(const LevelView&, const NoEdge<L>&, int, int) {
   return false;
 }
-__device__ __forceinline__ bool edge_node(const LevelView& v, const Edge2d& E, int x, int y) {
+__device__ __forceinline__ bool edge_node(const LevelView& v, const EdgeCount& E, int x, int y) {
   if (E.nb && ((!v.per[0] && (x == 0 || x == v.n[0] - 1)) ||
                (!v.per[1] && (y == 0 || y == v.n[1] - 1))))
     return true;
@@ -189,44 +202,53 @@ __device__ __forceinline__ void edge_restrict(const LevelView& v, const RefF& R,
   y = pc(1, a == 0 ? rb : ra);
 }
 
-template <bool WIDE, class S, int COLL, int PAR, bool MOV>
+// Special node t (lanes included) of runs run0 .. run0 + runs - 1, parity par;
+// du: its velocity deviation goes there too, when given.
+template <bool WIDE, class S, int COLL, bool MOV>
 __device__ __forceinline__ void edge_update(const LevelView& v, float omega, const RefF& R,
-                                            const Edge2d& E) {
+                                            const Edge2d& E, int par, float* du, unsigned t,
+                                            int run0, int runs) {
   using L = D2Q9;
   constexpr int BL = WIDE ? 4 : 1, TL = WIDE ? 16 : 1;  // lanes per outer and TN node
-  // (32 bits: the host keeps the lanes of all special nodes below 2^31)
-  unsigned t = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) *
-                   (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
-  const int lane = (int)(t & 31);  // (blocks hold whole warps)
+  const int lane = (int)(t & 31);  // (t of a warp's first lane is a multiple of 32)
   // outer nodes of every run first, padded to whole warps
-  const unsigned bl = ((unsigned)E.nb * v.batch * BL + 31) & ~31u;
+  const unsigned bl = ((unsigned)E.nb * runs * BL + 31) & ~31u;
   int x, y, lanes, sub;
   float g[L::Q];
   unsigned run;
   if (t < bl) {
     const unsigned item = t / BL;
     run = item / max(E.nb, 1);
-    if (run >= (unsigned)v.batch) return;  // whole groups leave
+    if (run >= (unsigned)runs) return;  // whole groups leave
+    const int k = (int)(item - run * E.nb);
+    run += run0;
     lanes = BL;
     sub = lane & (BL - 1);
-    edge_rebuild<BL>(v, R, E, (int)run, (int)(item - run * E.nb), sub, 0xfu << (lane & 28), x, y,
-                     g);
+    edge_rebuild<BL>(v, R, E, (int)run, k, sub, 0xfu << (lane & 28), x, y, g);
   } else {
     t -= bl;
     const unsigned item = t / TL;
     run = item / max(E.nt, 1);
-    if (run >= (unsigned)v.batch || E.nt == 0) return;
+    if (run >= (unsigned)runs || E.nt == 0) return;
+    const int k = (int)(item - run * E.nt);
+    run += run0;
     lanes = TL;
     sub = lane & (TL - 1);
-    edge_restrict<TL, S>(v, R, E, (int)run, (int)(item - run * E.nt), sub, 0xffffu << (lane & 16),
-                         x, y, g);
+    edge_restrict<TL, S>(v, R, E, (int)run, k, sub, 0xffffu << (lane & 16), x, y, g);
   }
   S* fp = run_ptr<S>(v, (int)run);
   const NodeAddr ad = node_addr<L>(v, x, y, 0);
+  if (du != nullptr && sub == 0) {
+    float drho, u[3];
+    deviations<L>(g, R, drho, u[0], u[1], u[2]);
+    float* d = du + (long long)run * L::D * v.plane + ad.at(0, 0, 0);
+    d[0] = u[0];
+    d[v.plane] = u[1];
+  }
   collide_emit<L, COLL, MOV>(g, omega, R, [&](auto I, float val) {
     constexpr int i = decltype(I)::value;
     if ((i & (lanes - 1)) != sub) return;  // the lanes share the stores
-    if constexpr (PAR == 0)
+    if (par == 0)
       Store<S>::st(fp + (long long)opp<L>(i) * v.plane + v.es * ad.at(0, 0, 0), val);
     else
       Store<S>::st(
@@ -235,17 +257,26 @@ __device__ __forceinline__ void edge_update(const LevelView& v, float omega, con
 }
 
 // The special blocks' part of an update kernel; true in those blocks.
+template <class L, class S, int COLL, int PAR, bool MOV, class E>
+__device__ __forceinline__ bool edge_block(const LevelView&, float, const RefF&, const E&) {
+  return false;
+}
 template <class L, class S, int COLL, int PAR, bool MOV>
 __device__ __forceinline__ bool edge_block(const LevelView& v, float omega, const RefF& R,
-                                           const EdgeArg<L>& E) {
-  if constexpr (L::D == 2) {
-    if ((int)blockIdx.z < E.nz) {
-      if (E.wide)
-        edge_update<true, S, COLL, PAR, MOV>(v, omega, R, E);
-      else
-        edge_update<false, S, COLL, PAR, MOV>(v, omega, R, E);
-      return true;
-    }
-  }
-  return false;
+                                           const Edge2d& E) {
+  if ((int)blockIdx.z >= E.nz) return false;
+  // (blocks hold whole warps)
+  const unsigned t = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) *
+                         (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
+  edge_update<true, S, COLL, MOV>(v, omega, R, E, PAR, nullptr, t, 0, v.batch);
+  return true;
+}
+
+// The special nodes of a level update in a launch of their own, run by run.
+template <bool WIDE, class S, int COLL, bool MOV>
+__global__ void __launch_bounds__(64)
+    k_edges(LevelView v, float omega, RefF R, const __grid_constant__ Edge2d E, int par,
+            float* du) {
+  edge_update<WIDE, S, COLL, MOV>(v, omega, R, E, par, du,
+                                  blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y, 1);
 }

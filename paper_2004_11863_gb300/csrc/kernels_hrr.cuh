@@ -63,14 +63,15 @@ __device__ __forceinline__ void store_post_i(S* f, long long plane, const NodeAd
 
 // --------------------------------------------------------------- velocity
 // (hybrid collision: TN nodes are left to the restriction, which writes
-// their velocity; otherwise every active node)
-template <class L, class S>
-__global__ void k_velocity(LevelView v, float* du, int par, RefF ref) {
+// their velocity; otherwise every active node but the special ones of a 2D
+// level, whose velocity k_edges has written)
+template <class L, class S, class EG>
+__global__ void k_velocity(LevelView v, float* du, int par, RefF ref, EG E) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int run = blockIdx.y;
   int x, y, z;
   if (!node_of(v, t, x, y, z)) return;
-  if (inactive(v, x, y, z) || (v.hrr && tn_node(v, x, y, z))) return;
+  if (inactive(v, x, y, z) || (v.hrr && tn_node(v, x, y, z)) || edge_node(v, E, x, y)) return;
   const S* f = run_cptr<S>(v, run);
   const NodeAddr a = node_addr<L>(v, x, y, z);
   float g[L::Q], drho, u[3];

@@ -16,8 +16,9 @@
 // The coarse level therefore streams and collides in one fused pass after
 // the fine sub-steps: nothing it streams is changed by the fine sub-steps
 // except its TN nodes, which the restriction rebuilds anyway.
-// In 2D the updates rebuild their own special nodes (kernels_edge.cuh): a step
-// is capture, advance(l+1), K1, advance(l+1), without K3 and K4.
+// In 2D one launch rebuilds and collides the nodes of K3 and K4, that of K1
+// itself or one beside it (kernels_edge.cuh): a step is capture, advance(l+1),
+// K1, advance(l+1).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -617,11 +618,13 @@ inline float omega_of(double tau) { return (float)(1.0 - 1.0 / tau); }
 // Sensors of level l for the update of parity par, once its pre-collision
 // state is final (kind 8; with_velocity: issue the velocity pass first,
 // which the hybrid schedule has already done).
-int sensor_pass(lbm_ctx* h, int l, int par, bool launch, bool with_velocity) {
+int sensor_pass(lbm_ctx* h, int l, int par, bool launch, bool with_velocity,
+                const EdgeCount& skip = EdgeCount{}) {
   Level& v = h->lev[l];
   if (!v.sens_on) return LBM_OK;
   float* du = (float*)v.du_mem;
-  if (with_velocity) LAUNCH_K(5, l, h->ops.velocity(v.view, h->cfg.storage, par, du, h->ref, h->cur));
+  if (with_velocity)
+    LAUNCH_K(5, l, h->ops.velocity(v.view, h->cfg.storage, par, du, h->ref, skip, h->cur));
   LAUNCH_K(8, l, h->ops.sensors(v.view, h->cfg.storage, du, par, v.sens, h->ref, h->cur));
   return LBM_OK;
 }
@@ -637,30 +640,9 @@ int read_slot(const Level& v, const float* wt) {
   return wt == kTimeDirect ? v.head : (v.head + 1) % 3;
 }
 
-// Lanes of special nodes when each takes several (an upper bound).
-constexpr long long EDGE_WIDE_MAX = 1LL << 20;
-
-// Whether level updates of this run take their special nodes along
-// (kernels_edge.cuh): 2D, not the hybrid collision, within the launch limits
-// on every level.
-bool edges_usable(const lbm_ctx* h) {
-  if (h->D != 2 || h->cfg.collision == LBM_HRR) return false;
-  for (int l = 0; l < h->nlev; ++l) {
-    const Level& v = h->lev[l];
-    long long items = l >= 1 ? v.bnd.count : 0;
-    if (l + 1 < h->nlev) items += h->lev[l + 1].tn.count;
-    const long long lanes = items * h->batch + EDGE_WIDE_MAX;
-    // (a slice of the update's grid holds at least 16 lanes per row)
-    if (lanes >= (1LL << 30) || lanes / (16LL * v.n[1]) + 1 + h->batch > 65535) return false;
-  }
-  return true;
-}
-
-bool any_sensors(const lbm_ctx* h) {
-  for (int l = 0; l < h->nlev; ++l)
-    if (h->lev[l].sens_on) return true;
-  return false;
-}
+// Whether the special nodes of this run's levels are rebuilt and collided in
+// one go (kernels_edge.cuh): 2D, not the hybrid collision.
+bool edges_usable(const lbm_ctx* h) { return h->D == 2 && h->cfg.collision != LBM_HRR; }
 
 // Description of level l's special nodes for its next update.
 Edge2d edge_desc(const lbm_ctx* h, int l, const float* wt) {
@@ -711,23 +693,13 @@ Edge2d edge_desc(const lbm_ctx* h, int l, const float* wt) {
   return E;
 }
 
-// The level update of advance(): with sensors on, the special nodes were
-// rebuilt into the planes for the sensors to read; a 2D update takes them
-// along all the same, so that sensors change no bit of a run.
-cudaError_t update_op(lbm_ctx* h, int l, int par, const float* wt) {
-  const Level& v = h->lev[l];
-  if (edges_usable(h))
-    return h->ops.stream_collide_edges(v.view, h->cfg.collision, h->cfg.storage, par,
-                                       omega_of(v.tau), h->ref, v.k1_bx, v.k1_by,
-                                       edge_desc(h, l, wt), h->cur);
-  return h->ops.stream_collide(v.view, h->cfg.collision, h->cfg.storage, par, omega_of(v.tau),
-                               h->ref, v.k1_bx, v.k1_by, xf_of(h, l), h->cur);
-}
-
-// One step of level l of a 2D run whose updates take their special nodes
-// along: capture, child's first sub-step, this level's update (its TN nodes
-// read the child's state between its sub-steps), child's second sub-step --
-// one chain on one stream.
+// One step of level l of a 2D run: capture, child's first sub-step, this
+// level's special nodes and update (its TN nodes read the child's state between
+// its sub-steps), child's second sub-step.  Few special nodes go with the
+// update's launch: one chain on one stream.  More of them go beside it, on the
+// side stream: two launches of nodes that need nothing of one another.  With
+// sensors on, whose velocity pass reads the special nodes' velocity, they go
+// first and write it.
 int advance_edges(lbm_ctx* h, int l, const float* wt, bool launch) {
   Level& v = h->lev[l];
   const int st = h->cfg.storage;
@@ -741,12 +713,47 @@ int advance_edges(lbm_ctx* h, int l, const float* wt, bool launch) {
     int rc = advance_edges(h, l + 1, v.nsteps == 0 ? kTimeLin : kTimeQuad, launch);
     if (rc) return rc;
   }
+  const Edge2d E = edge_desc(h, l, wt);
+  const bool inside = !v.sens_on && edges_few(E, h->batch);
+  const bool own = !inside && E.nb + E.nt > 0;
+  cudaStream_t main = h->cur;
+  bool forked = false;
+  auto fork = [&]() {  // the launches that follow go to the side stream
+    if (!launch || h->profiling) return LBM_OK;
+    CK(cudaEventRecord(h->ev_fork[l], main));
+    CK(cudaStreamWaitEvent(h->side[l], h->ev_fork[l], 0));
+    h->cur = h->side[l];
+    forked = true;
+    return LBM_OK;
+  };
+  auto back = [&]() {  // ... and these to the first one again
+    if (forked) CK(cudaEventRecord(h->ev_join[l], h->side[l]));
+    h->cur = main;
+    return LBM_OK;
+  };
+  int rc = LBM_OK;
+  if (own && !v.sens_on) rc = fork();
+  if (rc) return rc;
+  if (own)
+    LAUNCH_K(2, l, h->ops.edges(v.view, h->cfg.collision, st, par, omega_of(v.tau), h->ref, E,
+                                v.sens_on ? (float*)v.du_mem : nullptr, h->cur));
+  if (own && !v.sens_on) rc = back();
+  // (the rest of a level with sensors needs nothing of its child's second
+  // sub-step)
+  if (v.sens_on && child) rc = fork();
+  if (!rc) rc = sensor_pass(h, l, par, launch, true, E);
+  if (rc) return rc;
   LAUNCH_K(0, l, h->ops.stream_collide_edges(v.view, h->cfg.collision, st, par, omega_of(v.tau),
-                                             h->ref, v.k1_bx, v.k1_by, edge_desc(h, l, wt),
-                                             h->cur));
+                                             h->ref, v.k1_bx, v.k1_by, E, inside, h->cur));
+  if (v.sens_on && child) rc = back();
+  if (rc) return rc;
   v.last = par;
   v.nsteps++;
-  return child ? advance_edges(h, l + 1, kTimeDirect, launch) : LBM_OK;
+  if (forked && !v.sens_on) CK(cudaStreamWaitEvent(main, h->ev_join[l], 0));
+  if (child) rc = advance_edges(h, l + 1, kTimeDirect, launch);
+  if (rc) return rc;
+  if (forked && v.sens_on) CK(cudaStreamWaitEvent(main, h->ev_join[l], 0));
+  return LBM_OK;
 }
 
 // One step of level l with its finer levels (see the file comment).
@@ -805,9 +812,8 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
     // no barrier before the child's next phase: nothing there reads or
     // writes this level's populations)
     const Phase upd{0, l, par, 0, {}, {}, 0.0f, omega_of(v.tau), 1};
-    LAUNCH_K(0, l, update_op(h, l, par, wt));
-    // (a 2D update reads the child's state between its sub-steps itself)
-    if (fork && edges_usable(h)) CK(cudaEventRecord(h->ev_restrict[l], h->side[l]));
+    LAUNCH_K(0, l, h->ops.stream_collide(v.view, h->cfg.collision, st, par, omega_of(v.tau), ref,
+                                         v.k1_bx, v.k1_by, xf_of(h, l), h->cur));
     if (fork) {
       CK(cudaEventRecord(h->ev_join[l], h->side[l]));
       h->cur = main;
@@ -825,7 +831,8 @@ int advance(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wait_be
   if (rs) return rs;
   if (launch && wait_before_update) CK(cudaStreamWaitEvent(h->cur, wait_before_update, 0));
   if (h->recording) h->recording->push_back(Phase{0, l, par, 0, {}, {}, 0.0f, omega_of(v.tau)});
-  LAUNCH_K(0, l, update_op(h, l, par, wt));
+  LAUNCH_K(0, l, h->ops.stream_collide(v.view, h->cfg.collision, st, par, omega_of(v.tau), ref,
+                                       v.k1_bx, v.k1_by, xf_of(h, l), h->cur));
   v.last = par;
   v.nsteps++;
   return LBM_OK;
@@ -875,7 +882,7 @@ int advance_hrr(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wai
     LAUNCH_K(3, l, h->ops.restrict_hrr(v.view, c.view, c.tn, st, resc, par, 1 - c.last, du,
                                        omega_of(v.tau), sig, hrr_ks(h, v.tau), ref, h->cur));
     if (fork) CK(cudaEventRecord(h->ev_restrict[l], h->side[l]));
-    LAUNCH_K(5, l, h->ops.velocity(v.view, st, par, du, ref, h->cur));
+    LAUNCH_K(5, l, h->ops.velocity(v.view, st, par, du, ref, EdgeCount{}, h->cur));
     rc = sensor_pass(h, l, par, launch, false);
     if (rc) return rc;
     if (launch && wait_before_update) CK(cudaStreamWaitEvent(h->cur, wait_before_update, 0));
@@ -891,7 +898,7 @@ int advance_hrr(lbm_ctx* h, int l, const float* wt, bool launch, cudaEvent_t wai
     if (rc) return rc;
     if (fork) CK(cudaStreamWaitEvent(main, h->ev_join[l], 0));
   } else {
-    LAUNCH_K(5, l, h->ops.velocity(v.view, st, par, du, ref, h->cur));
+    LAUNCH_K(5, l, h->ops.velocity(v.view, st, par, du, ref, EdgeCount{}, h->cur));
     int rs = sensor_pass(h, l, par, launch, false);
     if (rs) return rs;
     if (launch && wait_before_update) CK(cudaStreamWaitEvent(h->cur, wait_before_update, 0));
@@ -928,10 +935,10 @@ int probe_launch(lbm_ctx* h, bool launch) {
 
 int coarse_step(lbm_ctx* h, bool launch) {
   // (the fused step's programs are recorded from the per-operation schedule)
-  int rc = h->cfg.collision == LBM_HRR        ? advance_hrr(h, 0, nullptr, launch, nullptr, false)
-           : !h->recording && !any_sensors(h) && edges_usable(h)
+  int rc = h->cfg.collision == LBM_HRR ? advance_hrr(h, 0, nullptr, launch, nullptr, false)
+           : edges_usable(h) && !h->recording
                ? advance_edges(h, 0, nullptr, launch)
-                                              : advance(h, 0, nullptr, launch, nullptr);
+               : advance(h, 0, nullptr, launch, nullptr);
   if (rc) return rc;
   return probe_launch(h, launch);
 }

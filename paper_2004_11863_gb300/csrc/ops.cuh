@@ -17,10 +17,14 @@ struct Ops {
   cudaError_t (*stream_collide)(const LevelView& v, int coll, int storage, int par, float omega,
                                 const RefState& ref, int bx, int by, const void* xf,
                                 cudaStream_t s);
-  // K1 of a 2D level with its rebuilt outer nodes and TN nodes.
+  // K1 of a 2D level with its rebuilt outer nodes and TN nodes (inside), or of
+  // its other nodes only.
   cudaError_t (*stream_collide_edges)(const LevelView& v, int coll, int storage, int par,
                                       float omega, const RefState& ref, int bx, int by,
-                                      const Edge2d& E, cudaStream_t s);
+                                      const Edge2d& E, bool inside, cudaStream_t s);
+  // Those nodes by themselves; du: their velocity deviations go there, or null.
+  cudaError_t (*edges)(const LevelView& v, int coll, int storage, int par, float omega,
+                       const RefState& ref, const Edge2d& E, float* du, cudaStream_t s);
   // K2: history capture (mode 0) or set-up (mode 1).
   cudaError_t (*capture)(const LevelView& p, const RingDesc& R, int storage, int par, int mode,
                          int s_new, int s_also, const TimeInt& ti, const RefState& ref,
@@ -36,8 +40,9 @@ struct Ops {
   // Hybrid collision (H-RR): velocity planes, the level update with
   // finite-difference strain, the parent strain history, the child's outer
   // layer collision and the restriction that collides TN nodes.
+  // (velocity: but for the special nodes of a 2D level, where E counts any)
   cudaError_t (*velocity)(const LevelView& v, int storage, int par, float* du, const RefState& ref,
-                          cudaStream_t s);
+                          const EdgeCount& E, cudaStream_t s);
   cudaError_t (*stream_collide_hrr)(const LevelView& v, int storage, int par, float omega,
                                     const float* du, float sig, float ks, const RefState& ref,
                                     cudaStream_t s);

@@ -28,20 +28,14 @@ RefF make_ref_f(const RefState& r) {
 
 // Prepends the z-slices of special blocks to a 2D update's grid
 // (kernels_edge.cuh).  First in the grid, so that their longer chain of loads
-// runs beside the plain blocks and not after them.  Several lanes a node up
-// to EDGE_WIDE_LANES of them, about what the GPU holds beside the plain
-// blocks (kernels_edge.cuh has both sides measured).
-template <class L>
-NoEdge<L> with_slices(const NoEdge<L>& E, int, dim3&, const dim3&) {
-  return E;
+// runs beside the plain blocks and not after them.
+template <class E>
+E with_slices(const E& e, int, dim3&, const dim3&) {
+  return e;
 }
-#ifndef EDGE_WIDE_LANES
-#define EDGE_WIDE_LANES 65536
-#endif
 inline Edge2d with_slices(Edge2d E, int batch, dim3& grid, const dim3& block) {
-  E.wide = (4LL * E.nb + 16LL * E.nt) * batch <= EDGE_WIDE_LANES;
-  const long long bl = ((long long)E.nb * batch * (E.wide ? 4 : 1) + 31) / 32 * 32;
-  const long long lanes = bl + (long long)E.nt * batch * (E.wide ? 16 : 1);
+  const long long bl = (4LL * E.nb * batch + 31) / 32 * 32;
+  const long long lanes = bl + 16LL * E.nt * batch;
   const long long slice = (long long)grid.x * grid.y * block.x * block.y;
   E.nz = (int)((lanes + slice - 1) / slice);
   grid.z += E.nz;
@@ -57,16 +51,16 @@ dim3 plane_blocks(const LevelView& v, int bx, int by, int nodes) {
   return dim3((v.n[0] + bx - 1) / bx, (v.n[1] + by * nodes - 1) / (by * nodes));
 }
 
-template <class L, class S, int COLL>
+template <class L, class S, int COLL, class EG>
 cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx,
-                         int by, const S* xf, const EdgeArg<L>& E, cudaStream_t s) {
+                         int by, const S* xf, const EG& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   if (v.run_stride >= (1LL << 31)) return cudaErrorInvalidValue;  // (32-bit offsets)
   dim3 block(bx, by, 1);
   const dim3 xy = plane_blocks<L>(v, bx, by, 2);
   dim3 grid(xy.x, xy.y,
             (v.n[2] + K1X2Pfz<L, S>::PZ - 1) / K1X2Pfz<L, S>::PZ * v.batch);
-  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
+  const EG Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   auto go = [&](auto M, auto X) {
@@ -98,9 +92,9 @@ cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefStat
   return cudaGetLastError();
 }
 
-template <class L, class S, int COLL>
+template <class L, class S, int COLL, class EG>
 cudaError_t sc_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx, int by,
-                      const S* xf, const EdgeArg<L>& E, cudaStream_t s) {
+                      const S* xf, const EG& E, cudaStream_t s) {
   // (the two-node update addresses a run with 32-bit offsets: larger runs
   // take the one-node update)
   if constexpr ((std::is_same<S, float>::value && K1X2Tune<L>::ON) ||
@@ -114,7 +108,7 @@ cudaError_t sc_launch(const LevelView& v, int par, float omega, const RefState& 
   }
   dim3 block(bx, by, 1);
   dim3 grid((v.n[0] + bx - 1) / bx, (v.n[1] + by * NPT - 1) / (by * NPT), v.n[2] * v.batch);
-  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
+  const EG Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   if (mov) {
@@ -131,14 +125,14 @@ cudaError_t sc_launch(const LevelView& v, int par, float omega, const RefState& 
   return cudaGetLastError();
 }
 
-template <class L, int COLL>
+template <class L, int COLL, class EG>
 cudaError_t sc_pair_launch(const LevelView& v, int par, float omega, const RefState& ref, int bx,
-                           int by, const __half* xf, const EdgeArg<L>& E, cudaStream_t s) {
+                           int by, const __half* xf, const EG& E, cudaStream_t s) {
   if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 128) return cudaErrorInvalidValue;
   dim3 block(bx, by, 1);
   dim3 grid = plane_blocks<L>(v, bx, by, 1);
   grid.z = v.n[2] * ((v.batch + 1) / 2);
-  const EdgeArg<L> Eg = with_slices(E, v.batch, grid, block);
+  const EG Eg = with_slices(E, v.batch, grid, block);
   const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
   const RefF R = make_ref_f<L>(ref);
   if (mov) {
@@ -155,9 +149,9 @@ cudaError_t sc_pair_launch(const LevelView& v, int par, float omega, const RefSt
   return cudaGetLastError();
 }
 
-template <class L, class S>
+template <class L, class S, class EG>
 cudaError_t sc_coll(const LevelView& v, int coll, int par, float omega, const RefState& ref,
-                    int bx, int by, const void* xf, const EdgeArg<L>& E, cudaStream_t s) {
+                    int bx, int by, const void* xf, const EG& E, cudaStream_t s) {
   const S* xs = static_cast<const S*>(xf);
   if (std::is_same<S, __half>::value && v.es == 2) {
     const __half* xh = static_cast<const __half*>(xf);
@@ -178,19 +172,60 @@ template <class L>
 cudaError_t stream_collide(const LevelView& v, int coll, int storage, int par, float omega,
                            const RefState& ref, int bx, int by, const void* xf,
                            cudaStream_t s) {
-  return storage == 0 ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, xf, EdgeArg<L>{}, s)
-                      : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, xf, EdgeArg<L>{}, s);
+  return storage == 0 ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, xf, NoEdge<L>{}, s)
+                      : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, xf, NoEdge<L>{}, s);
 }
 
-// The 2D update with its special nodes (E.nb, E.nt of them per run).
+// The 2D update with its special nodes, or without (E.nb, E.nt of them per
+// run).  A level that has none takes the instance without their code.
 template <class L>
 cudaError_t stream_collide_edges(const LevelView& v, int coll, int storage, int par, float omega,
-                                 const RefState& ref, int bx, int by, const Edge2d& E,
+                                 const RefState& ref, int bx, int by, const Edge2d& E, bool inside,
                                  cudaStream_t s) {
-  if constexpr (L::D == 2)
-    return storage == 0
-               ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, nullptr, E, s)
-               : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, nullptr, E, s);
+  if constexpr (L::D == 2) {
+    auto go = [&](const auto& e) {
+      return storage == 0 ? sc_coll<L, float>(v, coll, par, omega, ref, bx, by, nullptr, e, s)
+                          : sc_coll<L, __half>(v, coll, par, omega, ref, bx, by, nullptr, e, s);
+    };
+    if (E.nb + E.nt == 0) return go(NoEdge<L>{});
+    return inside ? go(E) : go(static_cast<const EdgeCount&>(E));
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <class S, int COLL>
+cudaError_t edges_launch(const LevelView& v, int par, float omega, const RefState& ref,
+                         const Edge2d& E, float* du, cudaStream_t s) {
+  const RefF R = make_ref_f<D2Q9>(ref);
+  const bool mov = ref.U[0] != 0.0 || ref.U[1] != 0.0 || ref.U[2] != 0.0;
+  auto go = [&](auto W, auto M) {
+    constexpr bool WIDE = decltype(W)::value, MOV = decltype(M)::value;
+    const long long bl = ((long long)E.nb * (WIDE ? 4 : 1) + 31) / 32 * 32;
+    const dim3 grid(blocks_for(bl + (long long)E.nt * (WIDE ? 16 : 1), 64), v.batch);
+    k_edges<WIDE, S, COLL, MOV><<<grid, 64, 0, s>>>(v, omega, R, E, par, du);
+  };
+  auto moving = [&](auto W) { mov ? go(W, std::true_type{}) : go(W, std::false_type{}); };
+  if (edges_few(E, v.batch))
+    moving(std::true_type{});
+  else
+    moving(std::false_type{});
+  return cudaGetLastError();
+}
+
+template <class L>
+cudaError_t edges(const LevelView& v, int coll, int storage, int par, float omega,
+                  const RefState& ref, const Edge2d& E, float* du, cudaStream_t s) {
+  if constexpr (L::D == 2) {
+    auto go = [&](auto x) {
+      using S = decltype(x);
+      switch (coll) {
+        case 0: return edges_launch<S, 0>(v, par, omega, ref, E, du, s);
+        case 1: return edges_launch<S, 1>(v, par, omega, ref, E, du, s);
+        default: return edges_launch<S, 2>(v, par, omega, ref, E, du, s);
+      }
+    };
+    return storage == 0 ? go(float{}) : go(__half{});
+  }
   return cudaErrorInvalidValue;
 }
 
@@ -277,6 +312,7 @@ RstDesc rst_desc(const TnDesc& T) {
 template <class L>
 cudaError_t restrict_tn(const LevelView& p, const LevelView& c, const TnDesc& T, int storage,
                         float resc, int ppar, int cpar, const RefState& ref, cudaStream_t s) {
+  if constexpr (L::D == 2) return cudaErrorInvalidValue;  // (kernels_edge.cuh)
   if (T.count == 0) return cudaSuccess;
   const RstDesc J = rst_desc<L>(T);
   dim3 block(32, RstTile<L>::NW);
@@ -329,13 +365,20 @@ cudaError_t restrict_hrr(const LevelView& p, const LevelView& c, const TnDesc& T
 
 template <class L>
 cudaError_t velocity(const LevelView& v, int storage, int par, float* du, const RefState& ref,
-                     cudaStream_t s) {
+                     const EdgeCount& E, cudaStream_t s) {
   const long long n = (long long)v.n[0] * v.n[1] * v.n[2];
   dim3 grid(blocks_for(n, 128), v.batch);
-  if (storage == 0)
-    k_velocity<L, float><<<grid, 128, 0, s>>>(v, du, par, make_ref_f<L>(ref));
+  auto go = [&](const auto& e) {
+    using EG = std::decay_t<decltype(e)>;
+    if (storage == 0)
+      k_velocity<L, float, EG><<<grid, 128, 0, s>>>(v, du, par, make_ref_f<L>(ref), e);
+    else
+      k_velocity<L, __half, EG><<<grid, 128, 0, s>>>(v, du, par, make_ref_f<L>(ref), e);
+  };
+  if (L::D == 2 && E.nb + E.nt > 0)
+    go(E);
   else
-    k_velocity<L, __half><<<grid, 128, 0, s>>>(v, du, par, make_ref_f<L>(ref));
+    go(NoEdge<L>{});
   return cudaGetLastError();
 }
 
@@ -543,6 +586,7 @@ Ops make_ops() {
   o.d = L::D;
   o.stream_collide = detail::stream_collide<L>;
   o.stream_collide_edges = detail::stream_collide_edges<L>;
+  o.edges = detail::edges<L>;
   o.capture = detail::capture<L>;
   o.inject = detail::inject<L>;
   o.restrict_tn = detail::restrict_tn<L>;
