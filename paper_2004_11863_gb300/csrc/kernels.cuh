@@ -478,6 +478,18 @@ __global__ void __launch_bounds__(128, MOV ? K1Tune<L, S>::MINB_MOV
 #ifndef K1X2_MINB1_XF_D2Q9
 #define K1X2_MINB1_XF_D2Q9 K1X2_MINB1_D2Q9
 #endif
+// (the even D3Q19 update without a face buffer spills 136 to 160 bytes for it at
+// four blocks, none at three: a level of 192^3 nodes, both parities, 175 -> 167
+// us a step at rest, 183 -> 167 with a moving reference)
+#ifndef K1X2_MINB_BGK_D3Q19
+#define K1X2_MINB_BGK_D3Q19 3
+#endif
+#ifndef K1X2_MINB_BGK_D3Q27
+#define K1X2_MINB_BGK_D3Q27 K1X2_MINB_D3Q27
+#endif
+#ifndef K1X2_MINB_BGK_D2Q9
+#define K1X2_MINB_BGK_D2Q9 K1X2_MINB_D2Q9
+#endif
 #ifndef K1X2_MINB1_BGK_D3Q19
 #define K1X2_MINB1_BGK_D3Q19 3
 #endif
@@ -495,6 +507,7 @@ struct K1X2Tune<D2Q9> {
   static constexpr bool ON_H = K1X2H_D2Q9;
   static constexpr int MINB = K1X2_MINB_D2Q9;
   static constexpr int MINB1 = K1X2_MINB1_D2Q9;
+  static constexpr int MINB_BGK = K1X2_MINB_BGK_D2Q9;
   static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D2Q9;
   static constexpr int MINB1_XF = K1X2_MINB1_XF_D2Q9;
   static constexpr int MINB_H = K1X2H_MINB_D2Q9;
@@ -506,6 +519,7 @@ struct K1X2Tune<D3Q19> {
   static constexpr bool ON_H = K1X2H_D3Q19;
   static constexpr int MINB = K1X2_MINB_D3Q19;
   static constexpr int MINB1 = K1X2_MINB1_D3Q19;
+  static constexpr int MINB_BGK = K1X2_MINB_BGK_D3Q19;
   static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D3Q19;
   static constexpr int MINB1_XF = K1X2_MINB1_XF_D3Q19;
   static constexpr int MINB_H = K1X2H_MINB_D3Q19;
@@ -517,6 +531,7 @@ struct K1X2Tune<D3Q27> {
   static constexpr bool ON_H = K1X2H_D3Q27;
   static constexpr int MINB = K1X2_MINB_D3Q27;
   static constexpr int MINB1 = K1X2_MINB1_D3Q27;
+  static constexpr int MINB_BGK = K1X2_MINB_BGK_D3Q27;
   static constexpr int MINB1_BGK = K1X2_MINB1_BGK_D3Q27;
   static constexpr int MINB1_XF = K1X2_MINB1_XF_D3Q27;
   static constexpr int MINB_H = K1X2H_MINB_D3Q27;
@@ -648,7 +663,8 @@ __device__ __forceinline__ void stream_collide_x2_pair(const LevelView& v, float
 template <class L, class S, int COLL, int PAR, bool MOV, bool XF, class EG>
 __global__ void __launch_bounds__(128, !std::is_same<S, float>::value
                                            ? (PAR ? K1X2Tune<L>::MINB1_H : K1X2Tune<L>::MINB_H)
-                                       : PAR == 0  ? K1X2Tune<L>::MINB
+                                       : PAR == 0
+                                           ? (COLL == 0 ? K1X2Tune<L>::MINB_BGK : K1X2Tune<L>::MINB)
                                        : COLL == 0 ? K1X2Tune<L>::MINB1_BGK
                                        : XF        ? K1X2Tune<L>::MINB1_XF
                                                    : K1X2Tune<L>::MINB1)
