@@ -15,9 +15,7 @@ namespace mlbm {
 // moves a node's population of both runs (plane and run_stride then count
 // the interleaved elements).  Bounded axes carry a
 // one-node ghost skin (x = -1 and x = n[0] on bounded x; y and z likewise);
-// periodic axes wrap.  2D rows are padded to a multiple of 32 elements; 3D rows
-// to 8, and planes to whole 32-element lines (the 3D updates walk a plane's
-// elements, see plane_node).
+// periodic axes wrap.  Rows are padded as in plane_pitch.
 struct LevelView {
   void* f;
   long long plane;       // elements between consecutive planes of a run

@@ -34,6 +34,7 @@
 
 #include "desc.h"
 #include "lattice.cuh"
+#include "planes.h"
 
 namespace mlbm {
 
@@ -563,23 +564,16 @@ struct K1X2Pfz {
                                                            : K1X2_PFZ_F;
 };
 
-// Node (x, y) at element e of a 3D level's z-plane, counted from its first
-// node (the two-node update: of its even rows; the odd ones are the other
-// lane's).  The 3D updates walk a plane's elements, not its rows: a refined
-// level has 2 E + 1 nodes in a row, so rows cut into warps leave a warp of
-// one lane at the end of each (a ninth one for 257 nodes), and rows padded to
-// whole cache lines leave a line of one node.  3D rows are padded to whole
-// sectors only (build_view), and warps run across their ends; elements
-// between rows (ghost nodes, padding) are idle lanes (x >= n[0]).  One
+// The 3D updates walk a plane's elements from its first node on (plane_node; the
+// two-node update: of its even rows, the odd ones are the other lane's), not
+// its rows: a refined level has 2 E + 1 nodes in a row, so rows cut into warps
+// leave a warp of one lane at the end of each (a ninth one for 257 nodes), and
+// rows padded to whole cache lines leave a line of one node.  3D rows are
+// padded to eight elements only (plane_pitch), and warps run across their ends;
+// elements between rows (ghost nodes, padding) are idle lanes (x >= n[0]).  One
 // periodic level of 257 x 512 x 256 nodes (D3Q19) 868 -> 829 us, 193 x 192^2
 // (D3Q27) 285 -> 273, 161 x 160^2 in binary16 82 -> 76; 256- and 192-node
 // rows as before.
-__device__ __forceinline__ void plane_node(const LevelView& v, unsigned e, int& x, int& y) {
-  const unsigned r = e / (unsigned)v.SX;
-  y = (int)r;
-  x = (int)(e - r * (unsigned)v.SX);
-}
-
 // Whether a lane of the warp lies on a face normal to x.
 __device__ __forceinline__ bool warp_has_xface(const LevelView& v, int x) {
   return __any_sync(__activemask(), x == 0 || x == v.n[0] - 1);
@@ -680,7 +674,7 @@ __global__ void __launch_bounds__(128, !std::is_same<S, float>::value
   }
   int x, y0;
   if constexpr (L::D == 3) {
-    plane_node(v, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y0);
+    plane_node(v.SX, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y0);
     y0 *= 2;
   } else {
     x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -736,9 +730,9 @@ template <class L, int COLL, bool MOV, bool XF>
 __global__ void __launch_bounds__(128, (L::Q == 27 ? K1EH_MINB_D3Q27 : K1EH_MINB_D3Q19) -
                                            (COLL == 0 ? 1 : 0))
     k_stream_collide_even_h(LevelView v, float omega, RefF R, const __half* __restrict__ xf) {
-  const unsigned e = (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
-  const unsigned hx = (unsigned)v.SX / 2, row = e / hx;
-  const int x = 2 * (int)(e - row * hx), y = (int)row;
+  int x, y;
+  plane_node(v.SX / 2, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y);
+  x *= 2;
   int z = blockIdx.z, run = 0;
   if (v.batch > 1) {
     run = z / v.n[2];
@@ -822,7 +816,7 @@ __global__ void __launch_bounds__(128, COLL == 0 ? K1PairTune<L>::MINB : K1PairT
   if (edge_block<L, __half, COLL, PAR, MOV>(v, omega, R, E)) return;
   int x, y;
   if constexpr (L::D == 3) {
-    plane_node(v, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y);
+    plane_node(v.SX, (blockIdx.x * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x, x, y);
   } else {
     x = blockIdx.x * blockDim.x + threadIdx.x;
     y = blockIdx.y * blockDim.y + threadIdx.y;

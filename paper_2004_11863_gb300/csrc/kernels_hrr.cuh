@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(128)
     k_stream_collide_hrr(LevelView v, float omega, RefF R, const float* du, float sig, float ks) {
   int x, y;
   if constexpr (L::D == 3) {
-    plane_node(v, blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x, x, y);
+    plane_node(v.SX, blockIdx.x * 128 + threadIdx.y * 32 + threadIdx.x, x, y);
   } else {
     x = blockIdx.x * 32 + threadIdx.x;
     y = blockIdx.y * 4 + threadIdx.y;

@@ -31,6 +31,7 @@
 
 #include "../../include/mlbm.h"
 #include "desc.h"
+#include "planes.h"
 #include "lattice.cuh"
 #include "ops.cuh"
 
@@ -85,7 +86,6 @@ struct Level {
   SensorState sens{};
 };
 
-int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Nodes per chunk of the host <-> device staging (lbm_init, lbm_macros):
 // two buffers of 4 doubles per node, 256 MB in all.
@@ -397,32 +397,13 @@ int build_layout(lbm_ctx* h) {
   return LBM_OK;
 }
 
-// Storage geometry (ghost skin on bounded axes).  Rows are padded to
-// MLBM_ROW_ALIGN elements in 2D; in 3D, whose updates walk the elements of a
-// plane (plane_node), to eight elements, with rows added until a plane is
-// whole 32-element lines -- unless that takes more memory than padded rows.
-#ifndef MLBM_ROW_ALIGN
-#define MLBM_ROW_ALIGN 32
-#endif
-#ifndef MLBM_ROW_ALIGN_3D
-#define MLBM_ROW_ALIGN_3D 8
-#endif
+// Storage geometry (ghost skin on bounded axes; rows as in plane_pitch).
 void build_view(lbm_ctx* h, int l) {
   Level& v = h->lev[l];
   LevelView& w = v.view;
   int g[3];
   for (int a = 0; a < 3; ++a) g[a] = v.per[a] ? 0 : 1;
-  w.SX = round_up(v.n[0] + 2 * g[0], MLBM_ROW_ALIGN);
-  w.SY = v.n[1] + 2 * g[1];
-  if (h->D == 3) {
-    const int sx = round_up(v.n[0] + 2 * g[0], MLBM_ROW_ALIGN_3D);
-    const int lines = sx % 32 == 0 ? 1 : sx % 16 == 0 ? 2 : sx % 8 == 0 ? 4 : 8;
-    const int sy = round_up(w.SY, lines);
-    if ((long long)sx * sy <= (long long)w.SX * w.SY) {
-      w.SX = sx;
-      w.SY = sy;
-    }
-  }
+  plane_pitch(h->D, v.n[0], v.n[1], g[0], g[1], w.SX, w.SY);
   const long long SZ = v.n[2] + 2 * g[2];
   w.off = 32 + ((long long)g[2] * w.SY + g[1]) * w.SX;
   long long need = w.off + SZ * w.SY * (long long)w.SX + 32;

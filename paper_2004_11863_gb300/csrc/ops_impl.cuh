@@ -47,7 +47,7 @@ inline Edge2d with_slices(Edge2d E, int batch, dim3& grid, const dim3& block) {
 template <class L>
 dim3 plane_blocks(const LevelView& v, int bx, int by, int nodes) {
   if (L::D == 3)
-    return dim3(blocks_for((long long)((v.n[1] + nodes - 1) / nodes - 1) * v.SX + v.n[0], bx * by));
+    return dim3(blocks_for(plane_elements(v.SX, v.n[0], (v.n[1] + nodes - 1) / nodes), bx * by));
   return dim3((v.n[0] + bx - 1) / bx, (v.n[1] + by * nodes - 1) / (by * nodes));
 }
 
@@ -68,7 +68,7 @@ cudaError_t sc_x2_launch(const LevelView& v, int par, float omega, const RefStat
     if constexpr (L::D == 3 && std::is_same<S, __half>::value) {
       // (rows, planes and runs of these levels start on even elements)
       if (par == 0 && v.es == 1 && v.SX % 2 == 0 && v.off % 2 == 0 && v.plane % 2 == 0) {
-        const long long pairs = (long long)(v.n[1] - 1) * (v.SX / 2) + (v.n[0] + 1) / 2;
+        const long long pairs = plane_elements(v.SX / 2, (v.n[0] + 1) / 2, v.n[1]);
         const dim3 eg(blocks_for(pairs, bx * by), 1, v.n[2] * v.batch);
         k_stream_collide_even_h<L, COLL, MOV, XF><<<eg, block, 0, s>>>(v, omega, R, xf);
         return;
