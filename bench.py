@@ -61,20 +61,28 @@ NCU_TRAFFIC = {
 
 
 def kernel_source_hash() -> str:
-    """Hash of the level update's source: lattice.cuh (the collisions) and
-    the part of kernels.cuh from the addressing helpers to the end of the
-    paired binary16 update.  Edits elsewhere do not void a
+    """Hash of the level update's source: lattice.cuh (the collisions),
+    planes.h (row pitch and walk), the part of kernels.cuh from the addressing
+    helpers to the end of the paired binary16 update, its launches in
+    ops_impl.cuh, and the layout in mlbm.cu.  Edits elsewhere do not void a
     traffic capture."""
     csrc = os.path.join(ROOT, "paper_2004_11863_gb300", "csrc")
     h = hashlib.sha256()
-    with open(os.path.join(csrc, "lattice.cuh"), "rb") as fh:
-        h.update(fh.read())
-    with open(os.path.join(csrc, "kernels.cuh"), "r") as fh:
-        k = fh.read()
-    start = k.index("__device__ __forceinline__ int wrapi")
-    end = k.index("k_stream_collide_pair(LevelView v")
-    end = k.index("\n}\n", end) + 3  # the end of k_stream_collide_pair
-    h.update(k[start:end].encode())
+
+    def part(name, first=None, last=None):
+        """From the text `first` to the end of the function `last`."""
+        with open(os.path.join(csrc, name)) as fh:
+            t = fh.read()
+        if first is not None:
+            t = t[t.index(first):]
+            t = t[:t.index("\n}\n", t.index(last)) + 3]
+        h.update(t.encode())
+
+    part("lattice.cuh")
+    part("planes.h")
+    part("kernels.cuh", "__device__ __forceinline__ int wrapi", "k_stream_collide_pair(LevelView v")
+    part("ops_impl.cuh", "dim3 plane_blocks(", "cudaError_t sc_pair_launch(")
+    part("mlbm.cu", "void build_view(", "void build_view(")
     return h.hexdigest()[:16]
 
 
@@ -187,6 +195,26 @@ def active_counts_oracle_free(case):
             N -= ina
         counts.append(N)
     return counts
+
+
+def special_nodes_2d(case, level):
+    """Nodes of a 2D level that are rebuilt from its parent or its child."""
+    lay = W.level_layout(case)
+    ring = lambda n, boxed: (int(np.prod(n))  # noqa: E731
+                             - int(np.prod([k - 2 * bool(b) for k, b in zip(n, boxed)])))
+    k = ring(lay[level]["n"][:2], lay[level]["boxed"][:2]) if level else 0
+    if level + 1 < len(lay):
+        (lo, hi), boxed = case.boxes[level], lay[level + 1]["boxed"]
+        k += ring([hi[a] - lo[a] - 1 if boxed[a] else lay[level]["n"][a] for a in range(2)],
+                  boxed[:2])
+    return k
+
+
+def updated_nodes(case, coll, counts, level, kt):
+    """Nodes that the update's launch takes: the active ones, but for those of
+    a 2D level that a launch of their own updates."""
+    own = case.dim == 2 and coll != "HRR" and f"inject_L{level}" in kt
+    return counts[level] - (special_nodes_2d(case, level) if own else 0)
 
 
 def dist_setup(args):
@@ -346,7 +374,7 @@ def workload_block(mlbm, case, storage, batch, stream, args, peak, collision=Non
     sb = 4 if storage == "fp32" else 2
     # algorithmic bytes of the level update: q populations read and written;
     # the hybrid update also reads the D velocity planes once
-    ab = counts[lev] * batch * (2 * case.q * sb + (4 * case.dim if coll == "HRR" else 0))
+    ab = updated_nodes(case, coll, counts, lev, kt) * batch * (2 * case.q * sb + (4 * case.dim if coll == "HRR" else 0))
     gbs = ab / (t_ms / n * 1e-3) / 1e9
     tot = sum(v[0] for v in kt.values())
     med = float(np.median(ms))
@@ -454,7 +482,8 @@ def main():
     dom_level = int(dom.split("_L")[1])
     t_ms, n = kt[dom]
     avg_s = t_ms / n * 1e-3
-    alg_bytes = counts[dom_level] * batch * 2 * case.q * s_bytes
+    alg_bytes = (updated_nodes(case, case.collision, counts, dom_level, kt) * batch * 2 * case.q
+                 * s_bytes)
     achieved = alg_bytes / avg_s / 1e9
     src_hash = kernel_source_hash()
     tr = NCU_TRAFFIC.get((case.name, args.storage, dom))

@@ -3,8 +3,8 @@
 //   k_stream_collide  fused stream + collide of every active node of a level
 //                     (eq. LBMequation), in place with the AA pattern;
 //   k_capture         parent pre-collision (drho, u, f^(1)) at t+1 on a child
-//                     box surface -> three-slot history (its first sub-step's state interpolated in time, eq.
-//                     TempInt);
+//                     box surface -> three-slot history, and the state at the
+//                     child's first sub-step (eq. TempInt);
 //   k_inject          child TF / IE nodes: spatial (eq. spaceInt)
 //                     interpolation staged per face tile in shared memory,
 //                     rescaling (eq. rescff), written where the child's next
@@ -25,9 +25,12 @@
 // reads g_i from plane opp(i) at n - xi_i and writes g_i* to plane i at
 // n + xi_i.  Every memory cell is read and then written by the same node, so
 // one array suffices.  The "read location" of (i, n) for parity p is where
-// the update of parity p fetches the pre-collision g_i(n); the interface
-// kernels overwrite exactly those cells for the nodes they rebuild, so the
-// level update itself has no special cases.
+// the update of parity p fetches the pre-collision g_i(n); k_inject,
+// k_inject_sep and k_restrict_tile overwrite exactly those cells for the nodes
+// they rebuild, so the 3D updates and those of the hybrid collision treat them
+// like any other (but for the face buffer below and the nodes the hybrid
+// collision takes elsewhere).  The other 2D updates leave these nodes to
+// kernels_edge.cuh.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -39,9 +42,6 @@
 namespace mlbm {
 
 __device__ __forceinline__ int wrapi(int x, int n) { return x < 0 ? x + n : (x >= n ? x - n : x); }
-
-// binary32 reference with its per-direction constants (formed on the host
-// by make_ref_f in the launch wrappers)
 
 // Element offsets of a node and of its 3^D neighbours inside a plane
 // (32-bit: the host keeps every plane below 2^31 elements; plane bases are
@@ -1641,6 +1641,20 @@ __global__ void __launch_bounds__(kDiagThreads)
     for (int j = 0; j < 3; ++j) partial[(long long)j * gridDim.x + blockIdx.x] = sh[j][0];
 }
 
+// rho and u of a node in FP64, moments to FP64 accuracy (moments_acc):
+// rho u = sum xi g + rho0 U.
+template <class L>
+__device__ __forceinline__ void fields_f64(const float (&g)[L::Q], const RefState& ref,
+                                           double (&o)[4]) {
+  double drho, jx, jy, jz;
+  moments_acc<L>(g, drho, jx, jy, jz);
+  const double r = ref.rho0 + drho, ri = 1.0 / r;
+  o[0] = r;
+  o[1] = (jx + ref.rho0 * ref.U[0]) * ri;
+  o[2] = (jy + ref.rho0 * ref.U[1]) * ri;
+  o[3] = L::D == 3 ? (jz + ref.rho0 * ref.U[2]) * ri : 0.0;
+}
+
 // rho and u (FP64) of the post-collision state; NaN at inactive nodes.
 template <class L, class S>
 // (nodes t0 .. t0 + cnt - 1 into rho[t - t0], u[a * us + t - t0])
@@ -1661,14 +1675,10 @@ __global__ void k_macros(LevelView v, int run, int last, double* rho, double* u,
   const NodeAddr a = node_addr<L>(v, x, y, z);
   float g[L::Q];
   load_post<L, S>(f, v.plane, a, last, v.es, g);
-  // moments to FP64 accuracy (moments_acc): rho u = sum xi g + rho0 U
-  double drho, jx, jy, jz;
-  moments_acc<L>(g, drho, jx, jy, jz);
-  const double r = ref.rho0 + drho, ri = 1.0 / r;
-  rho[k] = r;
-  u[k] = (jx + ref.rho0 * ref.U[0]) * ri;
-  u[us + k] = (jy + ref.rho0 * ref.U[1]) * ri;
-  u[2 * us + k] = L::D == 3 ? (jz + ref.rho0 * ref.U[2]) * ri : 0.0;
+  double o[4];
+  fields_f64<L>(g, ref, o);
+  rho[k] = o[0];
+  for (int c = 0; c < 3; ++c) u[c * us + k] = o[1 + c];
 }
 
 // The reference state as unevaluated sums of two binary32 numbers (rho0 and
@@ -1678,18 +1688,86 @@ struct RefPair {
   float m_hi[3], m_lo[3];
 };
 
+// a + b exactly: s rounded, e the rest (Knuth's TwoSum).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = a + b;
+  const float z = s - a;
+  e = (a - (s - z)) + (b - z);
+}
+
+// hi + lo rounded once (lo a few units in the last place of hi at most), rest:
+// what the rounding leaves.  True where an error of 2^-18 of lo could have
+// changed it (Ziv's test).
+__device__ __forceinline__ bool round_pair(float hi, float lo, float& out, float& rest) {
+  out = hi + lo;
+  rest = (hi - out) + lo;
+  return fmaf(rest, 1.0f + 0x1p-18f, out) != out;
+}
+
+// (nh + nl) / (rh + rl) rounded once, where it lies beside the midpoint between w
+// and the next number in the direction of rest: the sign of its difference to
+// the midpoint, times the divisor (exact there but for the products with rl).
+// True where the FP64 quotient, four roundings, may lie on the other side.
+__device__ __forceinline__ bool round_quotient(float nh, float nl, float rh, float rl, float& w,
+                                               float& rest) {
+  const int b = __float_as_int(w);
+  const float next = __int_as_float((rest > 0.0f) == (w > 0.0f) ? b + 1 : b - 1);
+  const float half = 0.5f * (next - w);
+  float rem, e;
+  two_sum(fmaf(-w, rh, nh), nl, rem, e);
+  const float beyond = fmaf(-half, rl, fmaf(-w, rl, fmaf(-half, rh, rem) + e));
+  if (beyond == 0.0f ? (b & 1) : (beyond > 0.0f) == (half > 0.0f)) {
+    w = next;
+    rest = -rest;
+  }
+  return rh != 1.0f && fabsf(beyond) <= 0x1p-50f * fabsf(nh);
+}
+
+// (x + rest) 2^-48 rounded once, x + rest a pair as above and the result
+// subnormal: x rounds to fewer bits, and where it lies halfway rest decides.
+__device__ __forceinline__ float subnormal_of(float x, float rest) {
+  const float y = x * 0x1p-48f, half = fmaf(-y, 0x1p48f, x);
+  const bool beyond = fabsf(half) == 0x1p-102f && rest != 0.0f && (rest > 0.0f) == (half > 0.0f);
+  return beyond ? y + copysignf(0x1p-149f, half) : y;
+}
+
+// Node t by way of FP64.  (Not inlined: the rare call's registers would be the
+// kernel's.)
+template <class L, class S>
+__device__ __noinline__ void macros_again(const LevelView& v, int run, int last, float* rho,
+                                          float* u, const RefState& ref, long long t) {
+  const long long N = (long long)v.n[0] * v.n[1] * v.n[2];
+  int x, y, z;
+  node_of(v, t, x, y, z);
+  float g[L::Q];
+  load_post<L, S>(run_cptr<S>(v, run), v.plane, node_addr<L>(v, x, y, z), last, v.es, g);
+  double o[4];
+  fields_f64<L>(g, ref, o);
+  rho[t] = (float)o[0];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[a * N + t] = (float)o[1 + a];
+}
+
 // rho and u of the post-collision state in binary32; NaN at inactive nodes.
-// The same values as k_macros rounded to binary32, without its FP64
-// arithmetic: every quantity stays an unevaluated binary32 pair (hi + lo, as
-// accurate as the sums of Acc2) until the one final rounding, and the
-// quotient is the rounded one plus its residual, formed exactly by an FMA,
-// over the density.  GB300 runs FP64 at a small fraction of its binary32
-// rate, so the FP64 reciprocal and products bounded the read-out: the
-// 67 M + 17 M nodes of a D3Q19 slab took 4.16 ms and take 1.40 ms (5.5 TB/s
-// of the 92 bytes a node; now bound by HBM).
+// The values of k_macros rounded to binary32, bit for bit, with its FP64
+// arithmetic only where that is in doubt: every quantity stays an unevaluated
+// binary32 pair (hi + lo) until the one final rounding, and the quotient is
+// the rounded one plus its residual, formed by an FMA, over the density.  The
+// pair is within 2^-20 units in the last place of the FP64 value, and where
+// that could change a rounding -- sums of a uniform far field and of binary16
+// storage lie halfway between two numbers, or next to it, often -- the exact
+// remainder decides (round_quotient).  FP64 (macros_again) is left with nodes
+// where its own roundings could, where the reference's momentum cancels the
+// node's, and whose numbers are far from one.
+// GB300 runs FP64 at a small fraction of its binary32 rate, so the FP64
+// reciprocal and products bounded the read-out: the 67 M + 17 M nodes of a
+// D3Q19 slab took 4.14 ms and take 1.92 ms (92 bytes a node; 1.68 ms without
+// the rounding's last step, bound by HBM, and off by a last bit at one node in
+// a thousand, by more where the reference's momentum cancels the node's).
 template <class L, class S>
 __global__ void __launch_bounds__(128)
-    k_macros_f(LevelView v, int run, int last, float* rho, float* u, RefPair R) {
+    k_macros_f(const __grid_constant__ LevelView v, int run, int last, float* rho, float* u,
+               const RefPair R, const __grid_constant__ RefState ref) {
   // A batch is read out in one launch per run and level; a launch that starts
   // only when the one before has drained costs 2.5 us of an idle GPU.  Here
   // the next one's blocks come up beside the last blocks of this one, and
@@ -1711,26 +1789,44 @@ __global__ void __launch_bounds__(128)
   load_post<L, S>(run_cptr<S>(v, run), v.plane, node_addr<L>(v, x, y, z), last, v.es, g);
   Acc2 r, m[3];
   moments_acc2<L>(g, r, m);
-  // rho = rho0 + drho as a pair (rh, rl): TwoSum, then one renormalisation
-  r.e += R.r_lo;
-  r.add(R.r_hi);
-  const float rh = r.s + r.e, rl = r.e - (rh - r.s);
-  rho[t] = rh;
+  // rho = rho0 + drho as a pair (rh, rl), exact where `lost` is zero
+  float h, l, c, lost, o[4], rest;
+  two_sum(R.r_hi, r.s, h, l);
+  two_sum(l, r.e, c, lost);
+  c += R.r_lo;
+  bool again = round_pair(h, c, o[0], rest) && (lost != 0.0f || R.r_lo != 0.0f);
+  const float rh = o[0];
+  // (in FP64 a density this near to one is one)
+  const float rl = rh == 1.0f && rest >= -0x1p-54f && rest <= 0x1p-53f ? 0.0f : rest;
+  // (also true of NaN)
+  again = again || !(rh >= 0x1p-20f && rh <= 0x1p20f && 4.0f * rh >= R.r_hi);
   const float inv = __frcp_rn(rh);
+  o[3] = 0.0f;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    float q = 0.0f;
-    if (a < L::D) {
+  for (int a = 0; a < L::D; ++a) {
+    // the momentum as a pair, times 2^48: no residual is subnormal
+    const bool moving = R.m_hi[a] != 0.0f;
+    if (moving) {
       m[a].e += R.m_lo[a];
       m[a].add(R.m_hi[a]);
-      const float nh = m[a].s + m[a].e, nl = m[a].e - (nh - m[a].s);
-      q = nh * inv;
-      const float d = (fmaf(-q, rh, nh) + fmaf(-q, rl, nl)) * inv;
-      // (no correction to an infinite or NaN quotient)
-      if (fabsf(q) < INFINITY) q += d;
     }
-    u[a * N + t] = q;
+    const float s48 = m[a].s * 0x1p48f, e48 = m[a].e * 0x1p48f;
+    const float nh = s48 + e48, nl = e48 - (nh - s48);
+    again = again || !(fabsf(nh) <= 0x1p68f) || (moving && fabsf(nh) < 0x1p46f * fabsf(R.m_hi[a]));
+    const float q = nh * inv;
+    const float d = (fmaf(-q, rh, nh) + fmaf(-q, rl, nl)) * inv;
+    float w;
+    if (round_pair(q, d, w, rest))
+      again = moving || round_quotient(nh, nl, rh, rl, w, rest) || again;
+    o[1 + a] = fabsf(w) < 0x1p-78f ? subnormal_of(w, rest) : w * 0x1p-48f;
   }
+  if (again) {
+    macros_again<L, S>(v, run, last, rho, u, ref, t);
+    return;
+  }
+  rho[t] = o[0];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[a * N + t] = o[1 + a];
 }
 
 // Post-collision populations shifted by the rest state, f_i - w_i rho0,

@@ -6,7 +6,8 @@
 // phase's items, and separates dependent phases by a grid barrier.  For
 // small runs, where a level update or an interface rebuild is a few
 // microseconds of work, this removes the per-kernel launch and drain cost of
-// the 7 (two levels) to 19 (three levels) launches of each coarse step.
+// the launches of each coarse step (two and three levels: 4 and 10 in 2D, 7
+// and 19 in 3D).
 //
 // The phases compute what the per-phase kernels compute, one item per
 // thread and without shared-memory staging (their launch shapes do not fit

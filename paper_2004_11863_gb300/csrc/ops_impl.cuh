@@ -529,8 +529,8 @@ cudaError_t macros_f(const LevelView& v, int storage, int run, int last, float* 
   c.stream = s;
   c.attrs = &at;
   c.numAttrs = 1;
-  return storage == 0 ? cudaLaunchKernelEx(&c, k_macros_f<L, float>, v, run, last, rho, u, R)
-                      : cudaLaunchKernelEx(&c, k_macros_f<L, __half>, v, run, last, rho, u, R);
+  return storage == 0 ? cudaLaunchKernelEx(&c, k_macros_f<L, float>, v, run, last, rho, u, R, ref)
+                      : cudaLaunchKernelEx(&c, k_macros_f<L, __half>, v, run, last, rho, u, R, ref);
 }
 
 template <class L>
