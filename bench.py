@@ -51,12 +51,12 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum on the fine-
     # level update of the same slab with full-width rows (257 fine nodes per
     # row) and y, z cut to 128 fine nodes (vortex3d_yz64, a 2-run batch,
-    # 8,421,376 node updates per launch): odd launches 668.5 + 604.3 and
-    # 668.4 + 601.4 MB, even 673.3 + 598.2 and 673.2 + 598.1 MB; per node
-    # update 151.1, 150.8, 151.0 and 151.0 B, mean 151.0 B (152 B
+    # 8,421,376 node updates per launch): odd launches 667.7 + 606.0 and
+    # 667.9 + 603.0 MB, even 672.9 + 598.5 and 672.9 + 598.0 MB; per node
+    # update 151.2, 150.9, 151.0 and 150.9 B, mean 151.0 B (152 B
     # algorithmic: the last writes of a launch are still in L2).  The rows,
     # and so the per-node traffic, are those of the full size.
-    ("vortex3d", "fp32", "update_L1"): {"bytes_per_node": 151.0, "src": "9c2143b7e8002aa1"},
+    ("vortex3d", "fp32", "update_L1"): {"bytes_per_node": 151.0, "src": "64796457dc4b0110"},
 }
 
 
